@@ -33,6 +33,18 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(
 
 struct DF2 { float2 h, l; };
 
+// Gather of one complex64 state value, 0 where !in (predicated, no branch).  The 64-byte prefetch size makes
+// L2 fetch the 64-byte blocks that hold a run of points instead of whole 128-byte lines (1.31x instead of
+// 1.64x the points' bytes on the oxide): this kernel is bound by that traffic, 330 -> 271 us for 512 oxide
+// rows.  The complex128 projection, bound by its arithmetic and latency, ran no faster with it (587 -> 609 us,
+// tile reduce included: the rest of the line is what the next lanes read) and keeps plain loads.
+__device__ __forceinline__ float2 ld_gather(const float2* p, bool in) {
+    float2 r = make_float2(0.f, 0.f);
+    asm("{ .reg .pred q; setp.ne.b32 q, %3, 0; @q ld.global.nc.L1::no_allocate.L2::64B.v2.f32 {%0, %1}, [%2]; }"
+        : "+f"(r.x), "+f"(r.y) : "l"(p), "r"((int)in));
+    return r;
+}
+
 // Ask L2 to start fetching a line a later chain will read (no register is held for it).
 __device__ __forceinline__ void prefetch_l2(const void* ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr)); }   // (re, im) pair of double-float numbers
 
@@ -168,7 +180,8 @@ __device__ __forceinline__ void proj_body_f32(const View& v, const Tile& t, int 
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
                 int i = i0 + c * Q;
-                x[c] = (i < t.np) ? __ldg(row + s_idx[i]) : make_float2(0.f, 0.f);
+                const bool in = i < t.np;
+                x[c] = ld_gather(row + (in ? s_idx[i] : 0), in);
             }
             if (G)
 #pragma unroll
@@ -472,8 +485,8 @@ __device__ __forceinline__ void proj_body_f32x2(const View& v, const Tile& t, in
                 const int i = i0 + c * Q;
                 const bool in = i < t.np;
                 const int g = in ? s_idx[i] : 0;
-                x0[c] = in ? __ldg(row0 + g) : make_float2(0.f, 0.f);
-                x1[c] = (in && row1) ? __ldg(row1 + g) : make_float2(0.f, 0.f);
+                x0[c] = ld_gather(row0 + g, in);
+                x1[c] = ld_gather(row1 + g, in && row1);
             }
             if (PF) {
                 // PF == 2: only the first and last lane of a band's group, whose points bound the Q
