@@ -138,29 +138,28 @@ cudaError_t launch_orbitals(const View& v, const double* radial_tab, const int* 
     return cudaGetLastError();
 }
 
-// S_{mm'} = dV sum_j phi_m phi_m' over the atom's points; one CTA per atom, fixed-order tree reduction.
+// S_{mm'} = dV sum_j phi_m phi_m' over the atom's points; one CTA per (atom, m m'), fixed-order tree reduction.
+// (All 25 sums of a d shell in one CTA, one after the other: 818 us for 16 atoms of 24405 and 11513 points, a
+// serial chain on 16 SMs; 60 us with a CTA each.)
 __global__ void k_overlap(View v, double* __restrict__ S) {
-    int a = blockIdx.x;
-    int M = v.atom_M[a];
-    int P = M * M;
+    const int a = blockIdx.x, pq = blockIdx.y;
+    const int M = v.atom_M[a];
+    if (pq >= M * M) return;
+    const int pm = pq / M, qm = pq % M;
     __shared__ double red[CTA];
-    for (int pq = 0; pq < P; ++pq) {
-        int pm = pq / M, qm = pq % M;
-        double acc = 0.0;
-        for (int t = v.atom_tile_beg[a]; t < v.atom_tile_end[a]; ++t) {
-            const Tile tl = v.tiles[t];
-            const double* ph = v.phi64 + tl.phi0;
-            for (int i = threadIdx.x; i < tl.np; i += blockDim.x) acc += ph[i * M + pm] * ph[i * M + qm];
-        }
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) S[a * MAXM * MAXM + pq] = red[0] * v.dV;
+    double acc = 0.0;
+    for (int t = v.atom_tile_beg[a]; t < v.atom_tile_end[a]; ++t) {
+        const Tile tl = v.tiles[t];
+        const double* ph = v.phi64 + tl.phi0;
+        for (int i = threadIdx.x; i < tl.np; i += blockDim.x) acc += ph[i * M + pm] * ph[i * M + qm];
+    }
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
+    if (threadIdx.x == 0) S[a * MAXM * MAXM + pq] = red[0] * v.dV;
 }
 
 // Cyclic Jacobi diagonalisation of the symmetric S (one thread per atom), then T = S^{-1/2} = U L^{-1/2} U^T
@@ -245,7 +244,7 @@ __global__ void k_lowdin_apply(View v, const double* __restrict__ T) {
 }
 
 cudaError_t launch_lowdin(const View& v, double* work_S, double* cond, cudaStream_t st) {
-    k_overlap<<<v.natoms, CTA, 0, st>>>(v, work_S);
+    k_overlap<<<dim3(v.natoms, v.maxM * v.maxM), CTA, 0, st>>>(v, work_S);
     k_inv_sqrt<<<(v.natoms + 63) / 64, 64, 0, st>>>(v, work_S, cond);
     k_lowdin_apply<<<v.ntiles, TILE, 0, st>>>(v, work_S);
     return cudaGetLastError();
