@@ -232,6 +232,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     c->canon_to_gpu.assign(natoms, {});
     c->atom_p0.resize(natoms); c->atom_phi0.resize(natoms);
     c->atom_umin.assign(natoms, std::vector<int>(3, 0));
+    c->atom_umax = c->atom_umin;
     std::vector<int> pt_idx, pt_u, seg_T;
     std::vector<int> seg_atom;
     c->tiles.clear();
@@ -268,7 +269,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
                 if (flags[box_off[a] + b] >= 0) canon_rank[b] = r++;
         }
         c->canon_to_gpu[a].assign(nin, 0);
-        int umin[3] = {1 << 30, 1 << 30, 1 << 30};
+        int umin[3] = {1 << 30, 1 << 30, 1 << 30}, umax[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
         int local = 0;
         for (int img = 0; img < NIMG; ++img) {
             const auto& L = by_img[img];
@@ -288,6 +289,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
                 pt_idx.push_back(idx);
                 pt_u.push_back(ix); pt_u.push_back(jy); pt_u.push_back(kz);
                 umin[0] = std::min(umin[0], ix); umin[1] = std::min(umin[1], jy); umin[2] = std::min(umin[2], kz);
+                umax[0] = std::max(umax[0], ix); umax[1] = std::max(umax[1], jy); umax[2] = std::max(umax[2], kz);
                 c->canon_to_gpu[a][canon_rank[b]] = local++;
             }
             int64_t len = (int64_t)pt_idx.size() - first;
@@ -319,7 +321,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
                 at += np;
             }
         }
-        for (int d = 0; d < 3; ++d) c->atom_umin[a][d] = umin[d];
+        for (int d = 0; d < 3; ++d) { c->atom_umin[a][d] = umin[d]; c->atom_umax[a][d] = umax[d]; }
         phi_off += nin * M;
     }
     c->MT = MT;

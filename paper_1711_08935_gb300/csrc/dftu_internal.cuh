@@ -161,7 +161,7 @@ struct Ctx {
     std::vector<Tile> tiles;
     std::vector<int> color_order;                  // tile indices grouped by colour
     std::vector<int> color_beg;                    // colour c is color_order[color_beg[c] .. color_beg[c+1])
-    std::vector<std::vector<int>> atom_umin;        // per atom minimum unfolded coordinate
+    std::vector<std::vector<int>> atom_umin, atom_umax;   // per atom smallest and largest unfolded coordinate
     int nspecies = 0, MT = 0, TM = 0, mat_total = 0;
     int64_t S = 0, phi_total = 0;
 
