@@ -494,8 +494,8 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = dalloc(c, &v.rho, (size_t)2 * mat);   // rho, then Pbar: one block for the sharded sums
     if (e == cudaSuccess) v.pbar = v.rho + mat;
     if (e == cudaSuccess) e = dalloc(c, &v.occ_part, (size_t)natoms * 2 * OCC_SPLIT * 2 * OCC_MAXP);
-    if (e == cudaSuccess) e = dalloc(c, &v.occ_count, (size_t)natoms * 2);
-    if (e == cudaSuccess) e = cudaMemset(v.occ_count, 0, (size_t)natoms * 2 * sizeof(int));
+    if (e == cudaSuccess) e = dalloc(c, &v.occ_count, (size_t)natoms * 2 + 1);
+    if (e == cudaSuccess) e = cudaMemset(v.occ_count, 0, ((size_t)natoms * 2 + 1) * sizeof(int));
     if (e == cudaSuccess) e = dalloc(c, &v.V, (size_t)mat);
     if (e == cudaSuccess) e = dalloc(c, &v.U, (size_t)natoms);
     if (e == cudaSuccess) e = dalloc(c, &v.J, (size_t)natoms);

@@ -110,7 +110,7 @@ struct View {
     double2* rho;          // per atom: collinear [ns][M][M]; non-collinear [2M][2M]   (rho = n^T)
     double2* pbar;         // same layout, renormalised (Eq. 8), transposed like rho
     double2* occ_part;     // [natoms][2][OCC_SPLIT][2][OCC_MAXP] partial rho / Pbar sums of the split CTAs
-    int* occ_count;        // [natoms][2] CTAs done per matrix; zero between launches
+    int* occ_count;        // [natoms][2] CTAs done per matrix, then atoms done by the U, J kernel; zero between launches
     double2* V;            // same layout, U_eff (1/2 - rho)
     const double* coul;
     const int* coul_set;   // [nspecies] 1 if set

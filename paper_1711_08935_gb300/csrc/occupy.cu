@@ -58,6 +58,7 @@ __device__ __forceinline__ void occupations_block(const View& v, const double* _
     const int kb0 = z * chunk, kb1 = min(total, kb0 + chunk);
     double2 r = make_double2(0.0, 0.0), pb = make_double2(0.0, 0.0);
     if (slice < SL) {
+#pragma unroll 4
         for (int kb = kb0 + slice; kb < kb1; kb += SL) {
             int k = kb / nbands, band = kb % nbands;
             double2 pa, pbv;
@@ -130,153 +131,159 @@ __device__ __forceinline__ double warp_sum(double x) {
     return x;
 }
 
-// Eqs. (10)-(11) [collinear/unpolarised] or (B5)-(B6) [non-collinear], then Eq. (3)/(A5) and Eq. (6).
-// One warp per atom (atoms warp0, warp0 + nw, ...); sums are lane-strided then tree-reduced (fixed order).
-__device__ __forceinline__ void acbn0_atoms(const View& v, int warp0, int nw) {
-    const int lane = threadIdx.x & 31;
-    for (int a = warp0; a < v.natoms; a += nw) {
-        const int M = v.atom_M[a], sp = v.atom_species[a];
-        const int64_t mo = v.atom_mat_off[a];
-        const double* Vc = v.coul + v.species_coul_off[sp];
-        const int M2 = M * M, M4 = M2 * M2;
-        double U, J, num_u = 0.0, num_j = 0.0, den_u = 0.0, den_j = 0.0;
-        const bool fixed = !isnan(v.fixU[a]);
-        if (!v.noncollinear) {
-            const int nchan = v.ns;   // stored channels; alpha = 0,1 maps to channel alpha % nchan
-            // paper's Pbar^alpha_{xy} = stored pbar[alpha][y][x]
-            if (!fixed) {
-                for (int e = lane; e < M4; e += 32) {
-                    int x = e / (M2 * M), y = (e / M2) % M, z = (e / M) % M, w = e % M;
-                    double vxyzw = Vc[((x * M + y) * M + z) * M + w];
-                    double vxwzy = Vc[((x * M + w) * M + z) * M + y];
-                    double2 Pt1 = make_double2(0, 0), Pt2 = make_double2(0, 0);
-                    for (int al = 0; al < 2; ++al) {
-                        int c = al % nchan;
-                        double2 p1 = v.pbar[mo + c * M2 + y * M + x], p2 = v.pbar[mo + c * M2 + w * M + z];
-                        Pt1.x += p1.x; Pt1.y += p1.y; Pt2.x += p2.x; Pt2.y += p2.y;
-                        num_j += (p1.x * p2.x - p1.y * p2.y) * vxwzy;
-                    }
-                    num_u += (Pt1.x * Pt2.x - Pt1.y * Pt2.y) * vxyzw;
-                }
-                num_u = warp_sum(num_u);
-                num_j = warp_sum(num_j);
-                double Nt[2] = {0, 0}, N2[2] = {0, 0};
-                for (int al = 0; al < 2; ++al) {
-                    int c = al % nchan;
-                    for (int m = 0; m < M; ++m) {
-                        double N = v.rho[mo + c * M2 + m * M + m].x;
-                        Nt[al] += N;
-                        N2[al] += N * N;
-                    }
-                }
-                double same = (Nt[0] * Nt[0] - N2[0]) + (Nt[1] * Nt[1] - N2[1]);
-                double opp = Nt[0] * Nt[1] + Nt[1] * Nt[0];
-                den_u = same + opp;
-                den_j = same;
-            }
-        } else {
-            const int D = 2 * M;
-            // paper's n^{st}_{xy} = stored rho[(t*M+y)][(s*M+x)]
-            auto PB = [&](int s, int t, int x, int y) { return v.pbar[mo + (t * M + y) * D + (s * M + x)]; };
-            auto NN = [&](int s, int t, int x) { return v.rho[mo + (t * M + x) * D + (s * M + x)]; };
-            if (!fixed) {
-                for (int e = lane; e < M4; e += 32) {
-                    int x = e / (M2 * M), y = (e / M2) % M, z = (e / M) % M, w = e % M;
-                    double vxyzw = Vc[((x * M + y) * M + z) * M + w];
-                    double vxwzy = Vc[((x * M + w) * M + z) * M + y];
-                    double2 d1 = make_double2(0, 0), d2 = make_double2(0, 0);
-                    for (int s = 0; s < 2; ++s) {
-                        double2 q1 = PB(s, s, x, y), q2 = PB(s, s, z, w);
-                        d1.x += q1.x; d1.y += q1.y; d2.x += q2.x; d2.y += q2.y;
-                        for (int t = 0; t < 2; ++t) {
-                            double2 r1 = PB(s, t, x, y), r2 = PB(t, s, z, w);
-                            num_j += (r1.x * r2.x - r1.y * r2.y) * vxwzy;
-                        }
-                    }
-                    num_u += (d1.x * d2.x - d1.y * d2.y) * vxyzw;
-                }
-                num_u = warp_sum(num_u);
-                num_j = warp_sum(num_j);
-                for (int s = 0; s < 2; ++s) {
-                    int o = 1 - s;
-                    for (int x = 0; x < M; ++x)
-                        for (int y = 0; y < M; ++y) {
-                            double2 ss_x = NN(s, s, x), ss_y = NN(s, s, y), oo_y = NN(o, o, y);
-                            double2 so_x = NN(s, o, x), os_y = NN(o, s, y);
-                            den_u += ss_x.x * oo_y.x - ss_x.y * oo_y.y;
-                            if (x != y) {
-                                double nss = ss_x.x * ss_y.x - ss_x.y * ss_y.y;
-                                den_u += nss;
-                                den_j += nss + (so_x.x * os_y.x - so_x.y * os_y.y);
-                            }
-                        }
-                    for (int x = 0; x < M; ++x) {
-                        double2 so = NN(s, o, x), os = NN(o, s, x);
-                        den_u -= so.x * os.x - so.y * os.y;
-                    }
-                }
-            }
-        }
-        bool zero = false;
-        if (fixed) {
-            U = v.fixU[a];
-            J = v.fixJ[a];
-        } else if (fabs(den_u) < 1e-14 || fabs(den_j) < 1e-14) {
-            U = 0.0; J = 0.0; zero = true;
-        } else {
-            U = num_u / den_u;
-            J = num_j / den_j;
-        }
-        const double Ue = U - J;
-        // Energy (Eq. 3 / A5): U_eff/2 sum_blocks (Tr n - Tr n^2); potential (Eq. 6): U_eff (1/2 - rho)
-        const int D = v.noncollinear ? 2 * M : M;
-        const int nblk = v.noncollinear ? 1 : v.ns;
-        double tr = 0.0;
-        for (int b = 0; b < nblk; ++b) {
-            const double2* R = v.rho + mo + (int64_t)b * D * D;
-            double part = 0.0;
-            for (int e = lane; e < D * D; e += 32) {
-                int x = e / D, y = e % D;
-                double2 rxy = R[x * D + y], ryx = R[y * D + x];
-                part -= rxy.x * ryx.x - rxy.y * ryx.y;
-                if (x == y) part += rxy.x;
-                double2 Vv = make_double2(Ue * ((x == y ? 0.5 : 0.0) - rxy.x), -Ue * rxy.y);
-                v.V[mo + (int64_t)b * D * D + e] = Vv;
-            }
-            tr += warp_sum(part);
-        }
-        if (!v.noncollinear && v.ns == 1) tr *= 2.0;
-        if (lane == 0) {
-            v.U[a] = U;
-            v.J[a] = J;
-            v.E[a] = 0.5 * Ue * tr;
-            if (zero) atomicOr(v.status, ST_ZERO_DENOM);
-        }
+constexpr int ACB_CTA = 128;   // threads per atom of the U, J kernel
+
+// Sums of N values per thread over the CTA, the same on every thread (fixed order: butterfly, then warps).
+template <int N>
+__device__ __forceinline__ void block_sum(double (&x)[N], double (*red)[ACB_CTA / 32]) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        x[i] = warp_sum(x[i]);
+        if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = x[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        x[i] = 0.0;
+        for (int w = 0; w < ACB_CTA / 32; ++w) x[i] += red[i][w];
     }
 }
 
-// E_U summed over atoms in atom order.
-__device__ __forceinline__ void energy_total(const View& v) {
-    double s = 0.0;
-    for (int a = 0; a < v.natoms; ++a) s += v.E[a];
-    v.Etot[0] = s;
-}
-
-constexpr int ACBN0_WARPS = 4;   // atoms per CTA of k_acbn0 (one warp each)
-
-__global__ void __launch_bounds__(32 * ACBN0_WARPS) k_acbn0(View v) {
-    acbn0_atoms(v, blockIdx.x * ACBN0_WARPS + (threadIdx.x >> 5), gridDim.x * ACBN0_WARPS);
-}
-
-__global__ void k_energy_total(View v) {
-    if (threadIdx.x == 0) energy_total(v);
-}
-
-__global__ void __launch_bounds__(256) k_acbn0_batch(const View* __restrict__ views) {
-    const View& v = views[blockIdx.x];
-    acbn0_atoms(v, threadIdx.x >> 5, blockDim.x >> 5);
+// Eqs. (10)-(11) [collinear/unpolarised] or (B5)-(B6) [non-collinear], then Eq. (3)/(A5) and Eq. (6).
+// One CTA per atom, its matrices in shared memory: the M^4 terms are FP64 work on one SM's narrow FP64 pipe, so
+// every atom gets an SM, and the loads are a single round (one warp per atom, four atoms to a CTA, matrices
+// read from memory term by term: 23 us and 3 us for the energy sum on 16 atoms; 12.5 us together).
+// The CTA that finishes last adds the atoms' energies (counter occ_count[2 natoms], zero between launches).
+__device__ __forceinline__ void acbn0_atom(const View& v, int a) {
+    __shared__ double2 s_rho[OCC_MAXP], s_pb[OCC_MAXP];
+    __shared__ double red[4][ACB_CTA / 32];
+    __shared__ int s_last;
+    const int tid = threadIdx.x;
+    const int M = v.atom_M[a], sp = v.atom_species[a];
+    const int64_t mo = v.atom_mat_off[a];
+    const double* Vc = v.coul + v.species_coul_off[sp];
+    const int M2 = M * M, M4 = M2 * M2;
+    const int D = v.noncollinear ? 2 * M : M;
+    const int nblk = v.noncollinear ? 1 : v.ns;
+    const int total = nblk * D * D;
+    for (int e = tid; e < total; e += ACB_CTA) { s_rho[e] = v.rho[mo + e]; s_pb[e] = v.pbar[mo + e]; }
+    const double fU = v.fixU[a], fJ = v.fixJ[a];
+    const bool fixed = !isnan(fU);
     __syncthreads();
-    if (threadIdx.x == 0) energy_total(v);
+    double U, J;
+    bool zero = false;
+    if (fixed) {
+        U = fU;
+        J = fJ;
+    } else {
+        double s4[4] = {0.0, 0.0, 0.0, 0.0};   // numerators of U and J, denominators of U and J
+        if (!v.noncollinear) {
+            const int nchan = v.ns;   // stored channels; alpha = 0,1 maps to channel alpha % nchan
+            // paper's Pbar^alpha_{xy} = stored pbar[alpha][y][x]
+            for (int e = tid; e < M4; e += ACB_CTA) {
+                const int x = e / (M2 * M), y = (e / M2) % M, z = (e / M) % M, w = e % M;
+                const double vxyzw = Vc[e], vxwzy = Vc[((x * M + w) * M + z) * M + y];
+                double2 Pt1 = make_double2(0, 0), Pt2 = make_double2(0, 0);
+                for (int al = 0; al < 2; ++al) {
+                    const int c = al % nchan;
+                    const double2 p1 = s_pb[c * M2 + y * M + x], p2 = s_pb[c * M2 + w * M + z];
+                    Pt1.x += p1.x; Pt1.y += p1.y; Pt2.x += p2.x; Pt2.y += p2.y;
+                    s4[1] += (p1.x * p2.x - p1.y * p2.y) * vxwzy;
+                }
+                s4[0] += (Pt1.x * Pt2.x - Pt1.y * Pt2.y) * vxyzw;
+            }
+            block_sum(s4, red);
+            double Nt[2] = {0, 0}, N2[2] = {0, 0};
+            for (int al = 0; al < 2; ++al) {
+                const int c = al % nchan;
+                for (int m = 0; m < M; ++m) {
+                    const double N = s_rho[c * M2 + m * M + m].x;
+                    Nt[al] += N;
+                    N2[al] += N * N;
+                }
+            }
+            const double same = (Nt[0] * Nt[0] - N2[0]) + (Nt[1] * Nt[1] - N2[1]);
+            s4[2] = same + (Nt[0] * Nt[1] + Nt[1] * Nt[0]);
+            s4[3] = same;
+        } else {
+            // paper's n^{st}_{xy} = stored rho[(t*M+y)][(s*M+x)]
+            auto PB = [&](int s, int t, int x, int y) { return s_pb[(t * M + y) * D + (s * M + x)]; };
+            auto NN = [&](int s, int t, int x) { return s_rho[(t * M + x) * D + (s * M + x)]; };
+            for (int e = tid; e < M4; e += ACB_CTA) {
+                const int x = e / (M2 * M), y = (e / M2) % M, z = (e / M) % M, w = e % M;
+                const double vxyzw = Vc[e], vxwzy = Vc[((x * M + w) * M + z) * M + y];
+                double2 d1 = make_double2(0, 0), d2 = make_double2(0, 0);
+                for (int s = 0; s < 2; ++s) {
+                    const double2 q1 = PB(s, s, x, y), q2 = PB(s, s, z, w);
+                    d1.x += q1.x; d1.y += q1.y; d2.x += q2.x; d2.y += q2.y;
+                    for (int t = 0; t < 2; ++t) {
+                        const double2 r1 = PB(s, t, x, y), r2 = PB(t, s, z, w);
+                        s4[1] += (r1.x * r2.x - r1.y * r2.y) * vxwzy;
+                    }
+                }
+                s4[0] += (d1.x * d2.x - d1.y * d2.y) * vxyzw;
+            }
+            for (int e = tid; e < 2 * M2; e += ACB_CTA) {   // (s, x, y); the spin-flip term once per (s, x)
+                const int s = e / M2, x = (e / M) % M, y = e % M, o = 1 - s;
+                const double2 ss_x = NN(s, s, x), ss_y = NN(s, s, y), oo_y = NN(o, o, y);
+                const double2 so_x = NN(s, o, x), os_y = NN(o, s, y);
+                s4[2] += ss_x.x * oo_y.x - ss_x.y * oo_y.y;
+                if (x != y) {
+                    const double nss = ss_x.x * ss_y.x - ss_x.y * ss_y.y;
+                    s4[2] += nss;
+                    s4[3] += nss + (so_x.x * os_y.x - so_x.y * os_y.y);
+                } else {
+                    s4[2] -= so_x.x * os_y.x - so_x.y * os_y.y;
+                }
+            }
+            block_sum(s4, red);
+        }
+        if (fabs(s4[2]) < 1e-14 || fabs(s4[3]) < 1e-14) {
+            U = 0.0; J = 0.0; zero = true;
+        } else {
+            U = s4[0] / s4[2];
+            J = s4[1] / s4[3];
+        }
+    }
+    const double Ue = U - J;
+    // Energy (Eq. 3 / A5): U_eff/2 sum_blocks (Tr n - Tr n^2); potential (Eq. 6): U_eff (1/2 - rho)
+    double tr[1] = {0.0};
+    for (int e = tid; e < total; e += ACB_CTA) {
+        const int eb = e % (D * D), x = eb / D, y = eb % D;
+        const double2 rxy = s_rho[e], ryx = s_rho[e - eb + y * D + x];
+        tr[0] -= rxy.x * ryx.x - rxy.y * ryx.y;
+        if (x == y) tr[0] += rxy.x;
+        v.V[mo + e] = make_double2(Ue * ((x == y ? 0.5 : 0.0) - rxy.x), -Ue * rxy.y);
+    }
+    block_sum(tr, red);
+    int* count = v.occ_count + 2 * v.natoms;
+    if (tid == 0) {
+        if (!v.noncollinear && v.ns == 1) tr[0] *= 2.0;
+        v.U[a] = U;
+        v.J[a] = J;
+        v.E[a] = 0.5 * Ue * tr[0];
+        if (zero) atomicOr(v.status, ST_ZERO_DENOM);
+        __threadfence();
+        s_last = (atomicAdd(count, 1) == v.natoms - 1);
+    }
+    __syncthreads();
+    if (!s_last || tid >= 32) return;
+    __threadfence();
+    double s = 0.0;
+    for (int i = tid; i < v.natoms; i += 32) s += __ldcg(v.E + i);
+    s = warp_sum(s);
+    if (tid == 0) {
+        v.Etot[0] = s;
+        *count = 0;
+    }
+}
+
+__global__ void __launch_bounds__(ACB_CTA) k_acbn0(View v) { acbn0_atom(v, blockIdx.x); }
+
+__global__ void __launch_bounds__(ACB_CTA) k_acbn0_batch(const View* __restrict__ views) {
+    const View& v = views[blockIdx.y];
+    if ((int)blockIdx.x < v.natoms) acbn0_atom(v, blockIdx.x);
 }
 
 // Hubbard forces (Sec. IV, state-gradient form, U_eff fixed): one CTA per (atom, direction),
@@ -412,10 +419,7 @@ cudaError_t launch_occupations(const View& v, const double* f, int nbands, cudaS
 }
 
 cudaError_t launch_acbn0(const View& v, cudaStream_t st) {
-    k_acbn0<<<(v.natoms + ACBN0_WARPS - 1) / ACBN0_WARPS, 32 * ACBN0_WARPS, 0, st>>>(v);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_energy_total<<<1, 32, 0, st>>>(v);
+    k_acbn0<<<v.natoms, ACB_CTA, 0, st>>>(v);
     return cudaGetLastError();
 }
 
@@ -430,7 +434,7 @@ cudaError_t launch_occupations_batch(const BatchLaunch& b, cudaStream_t st) {
 }
 
 cudaError_t launch_acbn0_batch(const BatchLaunch& b, cudaStream_t st) {
-    k_acbn0_batch<<<b.nsys, 256, 0, st>>>(b.views);
+    k_acbn0_batch<<<dim3(b.max_atoms, b.nsys), ACB_CTA, 0, st>>>(b.views);
     return cudaGetLastError();
 }
 
