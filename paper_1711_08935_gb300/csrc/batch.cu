@@ -210,7 +210,7 @@ dftu_status dftu_batch_occupations(dftu_batch b, dftu_stream stream) {
     cudaError_t e = launch_occupations_batch(b->L, reinterpret_cast<cudaStream_t>(stream));
     if (prev >= 0) cudaSetDevice(prev);
     if (e != cudaSuccess) return bfail(b, DFTU_ERR_CUDA, std::string("batch_occupations: ") + cudaGetErrorString(e));
-    for (auto* c : b->members) c->occ_ready = true;
+    for (auto* c : b->members) { c->occ_ready = true; c->last_stream = reinterpret_cast<cudaStream_t>(stream); }
     return DFTU_OK;
 }
 
@@ -229,7 +229,7 @@ dftu_status dftu_batch_acbn0_uj(dftu_batch b, dftu_stream stream) {
     cudaError_t e = launch_acbn0_batch(b->L, reinterpret_cast<cudaStream_t>(stream));
     if (prev >= 0) cudaSetDevice(prev);
     if (e != cudaSuccess) return bfail(b, DFTU_ERR_CUDA, std::string("batch_acbn0_uj: ") + cudaGetErrorString(e));
-    for (auto* c : b->members) c->pot_ready = true;
+    for (auto* c : b->members) { c->pot_ready = true; c->last_stream = reinterpret_cast<cudaStream_t>(stream); }
     return DFTU_OK;
 }
 

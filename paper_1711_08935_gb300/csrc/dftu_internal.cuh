@@ -163,6 +163,7 @@ struct Ctx {
     std::vector<int> color_beg;                    // colour c is color_order[color_beg[c] .. color_beg[c+1])
     std::vector<std::vector<int>> atom_umin, atom_umax;   // per atom smallest and largest unfolded coordinate
     int nspecies = 0, MT = 0, TM = 0, mat_total = 0;
+    int n_scalars = 0;   // doubles before rho in the results block (U, J, E, E_total)
     int64_t S = 0, phi_total = 0;
 
     View v{};
@@ -270,6 +271,9 @@ cudaError_t launch_apply_batch(const BatchLaunch& b, dftu_prec prec, dftu_f64_mo
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device, never inside a capture.
 bool smem_configured(const void* fn, int bytes);
+
+// SMs of the current device (looked up once per device).
+int sm_count();
 
 // Coulomb integrals of one atom's orbitals (blocking); W_out [P][P] with P = M(M+1)/2 pair index.
 int coulomb_atom(const View& v, const Ctx& c, int atom, double* V_dev, std::string& err);

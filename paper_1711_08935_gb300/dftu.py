@@ -362,20 +362,21 @@ class Handle:
         return [(self.ns, M) for M in self.M]
 
     def _unpack_mats(self, flat: np.ndarray):
-        out, o = [], 0
+        z, out, o = flat.view(np.complex128), [], 0
         for nb, D in self._mat_sizes():
             n = nb * D * D
-            out.append((flat[2 * o:2 * (o + n):2] + 1j * flat[2 * o + 1:2 * (o + n):2]).reshape(nb, D, D))
+            out.append(z[o:o + n].reshape(nb, D, D).copy())
             o += n
         return out
 
     def results(self, stream=None) -> dict:
-        tot = sum(nb * D * D for nb, D in self._mat_sizes())
-        n = np.zeros(2 * tot)
-        U, J, E = np.zeros(self.natoms), np.zeros(self.natoms), np.zeros(self.natoms)
-        Et = np.zeros(1)
-        self._check(self.lib.dftu_get_results(self.h, _dp(n), _dp(U), _dp(J), _dp(E), _dp(Et), _stream_ptr(stream, self.device)))
-        return dict(n=self._unpack_mats(n), U=U, J=J, EU_atom=E, EU=float(Et[0]))
+        tot, na = sum(nb * D * D for nb, D in self._mat_sizes()), self.natoms
+        x = np.empty(2 * tot + 3 * na + 1)   # n, U, J, E per atom, E
+        base, dp = x.ctypes.data, C.POINTER(C.c_double)
+        at = [C.cast(base + 8 * o, dp) for o in (0, 2 * tot, 2 * tot + na, 2 * tot + 2 * na, 2 * tot + 3 * na)]
+        self._check(self.lib.dftu_get_results(self.h, *at, _stream_ptr(stream, self.device)))
+        U, J, E = (x[2 * tot + i * na:2 * tot + (i + 1) * na].copy() for i in range(3))
+        return dict(n=self._unpack_mats(x[:2 * tot]), U=U, J=J, EU_atom=E, EU=float(x[-1]))
 
     def occupation_matrices(self, stream=None):
         tot = sum(nb * D * D for nb, D in self._mat_sizes())
