@@ -407,6 +407,47 @@ __device__ __forceinline__ void apply_project_body(const View& v, const Tile& t,
     }
 }
 
+// The bands of one group, band0 + (warp, lanes / Q), over the staged tile (coefficient table filled).
+template <int POL, int Q, int U, int PF, int G>
+__device__ __forceinline__ void apply_group(const View& v, const Tile& t, const ApplyArgs& a, int ks, int band0, int pe, bool fin, const int* s_idx,
+                                            const unsigned char* s_first, const unsigned char* after_idx, const unsigned char* after_c,
+                                            const unsigned char* s_gauge) {
+    static_assert(Q * U <= TILE_PAD - TILE, "batched loops read up to Q*U rows past the tile");
+    const int k = ks / v.ns, s = ks % v.ns;
+    const int lane = threadIdx.x & 31;
+    const int bl = (threadIdx.x >> 5) * (32 / Q) + lane / Q;
+    const int q = lane & (Q - 1);
+    const int band = band0 + bl;
+    const bool active = band < a.nbands;
+    const int64_t off = active ? (int64_t)k * a.sk + (int64_t)s * a.ss + (int64_t)band * a.sn : 0;
+    if constexpr (POL == A_F32PJ) {
+#define DFTU_PJ(MM, PR) apply_project_body<Q, MM, U, PF, PR>(v, t, a, off, q, bl, ks, band, active, s_idx, s_first, after_idx, after_c)
+        if (fin) {
+            switch (t.M) {
+                case 1: DFTU_PJ(1, 1); break;
+                case 3: DFTU_PJ(3, 1); break;
+                case 5: DFTU_PJ(5, 1); break;
+                default: DFTU_PJ(7, 1); break;
+            }
+        } else {
+            switch (t.M) {
+                case 1: DFTU_PJ(1, 0); break;
+                case 3: DFTU_PJ(3, 0); break;
+                case 5: DFTU_PJ(5, 0); break;
+                default: DFTU_PJ(7, 0); break;
+            }
+        }
+#undef DFTU_PJ
+    } else if (active) {
+        switch (t.M) {
+            case 1: apply_body<POL, Q, 1, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
+            case 3: apply_body<POL, Q, 3, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
+            case 5: apply_body<POL, Q, 5, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
+            default: apply_body<POL, Q, 7, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
+        }
+    }
+}
+
 // One work item: tile `tile_id` (a tile of the current colour) of the system (v, a), component ks, band chunk `chunk`.
 template <int POL, int Q, int NBG, int U, int PF, int G>
 __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, int tile_id, int ks, int chunk,
@@ -416,7 +457,7 @@ __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, in
     constexpr int BPW = 32 / Q;
     constexpr int BPC = (CTA / 32) * BPW;
     const Tile t = v.tiles[tile_id];
-    const int k = ks / v.ns, s = ks % v.ns;
+    const int k = ks / v.ns;
     const int M = t.M;
     unsigned char* after_idx = smem + TILE * sizeof(int);
     // coefficient table [BPC][MAXM] in 16-byte slots: double2 (F64), (hi.re, hi.im, lo.re, lo.im) (PAIR), float2 (F32)
@@ -469,9 +510,6 @@ __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, in
             for (int i = threadIdx.x; i < TILE_PAD; i += CTA)
                 reinterpret_cast<float4*>(s_gauge)[i] = (i < t.np) ? v.gauge_f[t.p0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const int lane = threadIdx.x & 31;
-    const int bl = (threadIdx.x >> 5) * BPW + lane / Q;
-    const int q = lane & (Q - 1);
     const int mo = v.atom_moff[t.atom];
     for (int g = 0; g < NBG; ++g) {
         const int band0 = (chunk * NBG + g) * BPC;
@@ -498,38 +536,13 @@ __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, in
             } else reinterpret_cast<float2*>(after_idx)[cb * MAXM + m] = make_float2((float)c.x, (float)c.y);
         }
         __syncthreads();
-        const int band = band0 + bl;
-        if constexpr (POL == A_F32PJ) {
-            const bool active = band < a.nbands;
-            const int64_t off = active ? (int64_t)k * a.sk + (int64_t)s * a.ss + (int64_t)band * a.sn : 0;
-            const int qq = lane & (Q - 1);
-#define DFTU_PJ(MM, PR) apply_project_body<Q, MM, U, PF, PR>(v, t, a, off, qq, bl, ks, band, active, s_idx, s_first, after_idx, after_c)
-            if (v.tile_final[tile_id]) {
-                switch (M) {
-                    case 1: DFTU_PJ(1, 1); break;
-                    case 3: DFTU_PJ(3, 1); break;
-                    case 5: DFTU_PJ(5, 1); break;
-                    default: DFTU_PJ(7, 1); break;
-                }
-            } else {
-                switch (M) {
-                    case 1: DFTU_PJ(1, 0); break;
-                    case 3: DFTU_PJ(3, 0); break;
-                    case 5: DFTU_PJ(5, 0); break;
-                    default: DFTU_PJ(7, 0); break;
-                }
-            }
-#undef DFTU_PJ
-        } else if (band < a.nbands) {
-            const int64_t off = (int64_t)k * a.sk + (int64_t)s * a.ss + (int64_t)band * a.sn;
-            const int pe = s_pe;
-            switch (M) {
-                case 1: apply_body<POL, Q, 1, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
-                case 3: apply_body<POL, Q, 3, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
-                case 5: apply_body<POL, Q, 5, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
-                default: apply_body<POL, Q, 7, U, PF, G>(t, a, off, q, bl, s_idx, s_first, after_idx, after_c, pe, s_gauge); break;
-            }
-        }
+        // a last group of at most half the bands takes twice the lanes per band (shorter chains, no idle warps)
+        const bool fin = POL == A_F32PJ && v.tile_final[tile_id];
+        constexpr bool TAIL = Q == 16 && NBG == 4 && PF == 1 && (POL == A_PAIR ? U == 4 : POL == A_F32P && U == 8);   // the default shapes (the fused one would spill)
+        if (TAIL && a.nbands - band0 <= BPC / 2)
+            apply_group<POL, TAIL ? 2 * Q : Q, TAIL ? 4 : U, PF, G>(v, t, a, ks, band0, s_pe, fin, s_idx, s_first, after_idx, after_c, s_gauge);
+        else
+            apply_group<POL, Q, U, PF, G>(v, t, a, ks, band0, s_pe, fin, s_idx, s_first, after_idx, after_c, s_gauge);
     }
 }
 
@@ -577,12 +590,20 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
     cudaError_t e = cudaSuccess;
     if (!smem_configured((const void*)fn, (int)smem)) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    // A colour with few tiles (where spheres overlap) or a small call leaves SMs idle with NBG groups of bands per
+    // CTA, and is then one chain of latencies: it takes one group of 32 lanes per band.  The update of a point
+    // does not depend on the shape.
+    auto small = k_apply<POL, 32, 1, 4, PF, G>;
+    if (!smem_configured((const void*)small, (int)smem)) e = cudaFuncSetAttribute(small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t slots = 3 * (int64_t)sm_count();
     for (size_t c = 0; c + 1 < color_beg.size(); ++c) {
         int n = color_beg[c + 1] - color_beg[c];
         if (n == 0) continue;
         a.tile_list = color_order + color_beg[c];
         dim3 grid(n, (a.nbands + BPC * NBG - 1) / (BPC * NBG), v.nk * v.ns);
-        fn<<<grid, CTA, smem, st>>>(v, a);
+        if ((int64_t)grid.x * grid.y * grid.z >= slots) fn<<<grid, CTA, smem, st>>>(v, a);
+        else small<<<dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st>>>(v, a);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
