@@ -121,7 +121,7 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
         return bfail(b, DFTU_ERR_INVALID_ARG, "batch_bind: null arrays or bad precision");
     const int n = (int)b->members.size();
     std::vector<ProjArgs> args(n);
-    int64_t max_reduce = 1;
+    int64_t max_reduce = 1, max_ctas = 1;
     int max_rows = 1;
     for (int s = 0; s < n; ++s) {
         Ctx* c = b->members[s];
@@ -140,6 +140,7 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
         }
         args[s] = a;
         max_reduce = std::max<int64_t>(max_reduce, (int64_t)c->nk * c->ns * nbands[s] * c->MT);
+        max_ctas = std::max<int64_t>(max_ctas, (int64_t)c->nk * c->ns * ((nbands[s] + 31) / 32) * (int64_t)c->atoms.size());
         max_rows = std::max(max_rows, (c->spin == DFTU_NONCOLLINEAR ? c->nk : c->nk * c->ns) * nbands[s] * c->nspecies);
     }
     int prev = -1;
@@ -155,6 +156,7 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
     b->L.args = b->d_args;
     b->L.f = b->d_f;
     b->L.max_reduce = max_reduce;
+    b->L.max_reduce_ctas = max_ctas;
     b->L.max_rows_nbar = max_rows;
     b->prec = prec;
     b->nbands.assign(nbands, nbands + n);

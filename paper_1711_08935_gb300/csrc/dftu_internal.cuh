@@ -202,6 +202,7 @@ struct BatchLaunch {
     int nsys;
     int maxM;
     int64_t max_reduce;       // max over systems of (k*spin rows) * nbands * sum M
+    int64_t max_reduce_ctas;  // max over systems of (k*spin rows) * band chunks of 32 * atoms (the tile reduce's CTAs)
     int max_rows_nbar;        // max over systems of rows * nbands * species (the Nbar threads)
     int max_atoms, max_ns;
 };
