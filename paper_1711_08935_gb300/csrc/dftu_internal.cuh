@@ -214,6 +214,8 @@ cudaError_t launch_sphere_flags(const View& v, const double* pos, const double* 
 cudaError_t launch_seg_phases(const View& v, cudaStream_t st);
 cudaError_t launch_orbitals(const View& v, const double* radial_tab, const int* radial_off,
                             const int* radial_nr, const double* radial_dr, cudaStream_t st);
+// S[atom][m][m'] (rows of MAXM*MAXM doubles, M x M used) = dV sum phi_m phi_m' of the current orbitals.
+cudaError_t launch_overlap(const View& v, double* S, cudaStream_t st);
 cudaError_t launch_lowdin(const View& v, double* work_S, double* cond, cudaStream_t st);
 
 constexpr int NVARIANTS = 8;   // shapes per streaming kernel (see dftu_set_kernel_variant)

@@ -243,8 +243,14 @@ __global__ void k_lowdin_apply(View v, const double* __restrict__ T) {
     }
 }
 
+cudaError_t launch_overlap(const View& v, double* S, cudaStream_t st) {
+    k_overlap<<<dim3(v.natoms, v.maxM * v.maxM), CTA, 0, st>>>(v, S);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_lowdin(const View& v, double* work_S, double* cond, cudaStream_t st) {
-    k_overlap<<<dim3(v.natoms, v.maxM * v.maxM), CTA, 0, st>>>(v, work_S);
+    cudaError_t e = launch_overlap(v, work_S, st);
+    if (e != cudaSuccess) return e;
     k_inv_sqrt<<<(v.natoms + 63) / 64, 64, 0, st>>>(v, work_S, cond);
     k_lowdin_apply<<<v.ntiles, TILE, 0, st>>>(v, work_S);
     return cudaGetLastError();
