@@ -499,7 +499,8 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = dalloc(c, &v.part, (size_t)3 * v.part_dir_stride);
     if (e == cudaSuccess) e = dalloc(c, &v.pgrad, (size_t)3 * rowsP * c->max_bands * MT);
     if (e == cudaSuccess) e = dalloc(c, &c->d_forces, (size_t)3 * natoms);
-    if (e == cudaSuccess) e = dalloc(c, &c->d_current, (size_t)3 * natoms);
+    if (e == cudaSuccess) e = dalloc(c, &c->d_current, (size_t)3 * CUR_SPLIT * natoms);
+    if (e == cudaSuccess) e = dalloc(c, &v.cur_A, (size_t)natoms * MAXM * CUR_MAXQ);
     if (e == cudaSuccess) e = dalloc(c, &c->d_fll, (size_t)2 * natoms);
     if (e == cudaSuccess) e = dalloc(c, &v.gauge_d, (size_t)c->S);
     if (e == cudaSuccess) e = dalloc(c, &v.gauge_f, (size_t)c->S);
@@ -529,7 +530,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = launch_orbitals(v, d_rtab, d_roff, d_rnr, d_rdr, 0);
     double* cond = work + (size_t)natoms * MAXM * MAXM;
     if (e == cudaSuccess) e = launch_lowdin(v, work, cond, 0);
-    if (e == cudaSuccess) e = launch_displaced_orbitals(v, phi_off, 0);
+    if (e == cudaSuccess) e = launch_current_tables(v, phi_off, work, d_rtab, d_roff, d_rnr, d_rdr, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(c, e, "setup_atoms: orbitals");
     // S^(-1/2) exists only for orbitals that are linearly independent on the sphere (Sec. III)
@@ -990,7 +991,7 @@ dftu_status dftu_hubbard_current(dftu_handle h, const void* psi, dftu_prec prec,
     if (!gpu_addressable(c->device, psi, st)) return fail(c, DFTU_ERR_INVALID_ARG, "hubbard_current: the states are not addressable by this GPU (device memory of another GPU, or pageable host memory on a device without pageable access)");
     if (!gpu_addressable(c->device, f, st)) return fail(c, DFTU_ERR_INVALID_ARG, "hubbard_current: f is not addressable by this GPU");
     const int64_t gstride = (int64_t)c->nk * c->ns * c->max_bands * c->MT;
-    View vq = c->v;   // the same states projected onto phi_m d_a (a = x, y, z) in one launch, into the gradient buffer
+    View vq = c->v;   // the same states projected onto the tables of the current in one launch, into the gradient buffer
     vq.phi64 = c->v.phid64;
     vq.phi_hi = c->v.phid_hi;
     vq.phi_lo = c->v.phid_lo;
@@ -998,10 +999,13 @@ dftu_status dftu_hubbard_current(dftu_handle h, const void* psi, dftu_prec prec,
     cudaError_t e = launch_project_dirs(vq, psi, prec, c->f64_mode, nbands, sk, ss, sn, c->gauge_on, c->v.pgrad, gstride, st);
     if (e == cudaSuccess) e = launch_current(c->v, f, nbands, c->d_current, st);
     const int na = (int)c->atoms.size();
-    std::vector<double> Jat(3 * (size_t)na);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(Jat.data(), c->d_current, Jat.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
+    std::vector<double> part(3 * CUR_SPLIT * (size_t)na), Jat(3 * (size_t)na, 0.0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(part.data(), c->d_current, part.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(c, e, "hubbard_current");
+    for (int a = 0; a < na; ++a)
+        for (int z = 0; z < CUR_SPLIT; ++z)
+            for (int d = 0; d < 3; ++d) Jat[3 * a + d] += part[3 * ((size_t)a * CUR_SPLIT + z) + d];
     if (J_atom_out) std::copy(Jat.begin(), Jat.end(), J_atom_out);
     if (J_out) {
         J_out[0] = J_out[1] = J_out[2] = 0.0;

@@ -627,7 +627,7 @@ cudaError_t launch_apply(const View& v, void* psi, dftu_prec prec, dftu_f64_mode
     if (gauge) {   // one shape per arithmetic policy with the gauge phases (Sec. V)
         if (prec == DFTU_C64) return run_apply<A_F32, 8, 4, 8, 1, 1>(v, a, color_order, color_beg, st);
         if (mode == DFTU_F64_NATIVE) return run_apply<A_F64, 8, 4, 4, 0, 1>(v, a, color_order, color_beg, st);
-        return run_apply<A_PAIR, 8, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
+        return run_apply<A_PAIR, 16, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
     }
 #define DFTU_CASE_F32(i, POL, Q, NBG, U, PF) case i: return run_apply<POL, Q, NBG, U, PF>(v, a, color_order, color_beg, st);
 #define DFTU_CASE_PAIR(i, Q, NBG, U, PF) case i: return run_apply<A_PAIR, Q, NBG, U, PF>(v, a, color_order, color_beg, st);

@@ -34,6 +34,15 @@ constexpr int OCC_MAXP = (2 * MAXM) * (2 * MAXM);   // largest matrix (non-colli
 constexpr double LOWDIN_MIN_RATIO = 1e-10;   // smallest accepted lambda_min / lambda_max of an atom's orbital
                                             // overlap; below it S^(-1/2) is refused (orbitals dependent)
 
+constexpr int CUR_MAXQ = 10;   // monomials of degree l <= 3
+constexpr int CUR_SPLIT = 8;   // CTAs sharing an atom's sum over states of the current
+
+// Monomials of degree D are numbered t(t+1)/2 + k for x^(D-t) y^(t-k) z^k, whatever D: multiplying by x keeps the
+// number, by y or z moves it to the next t.
+__host__ __device__ constexpr int cur_functions(int M) { return ((M - 1) / 2 + 2) * ((M - 1) / 2 + 3) / 2; }   // degree l + 1
+__host__ __device__ constexpr int cur_monomials(int M) { return ((M - 1) / 2 + 1) * ((M - 1) / 2 + 2) / 2; }   // degree l
+__host__ __device__ constexpr int cur_tables(int M) { return (cur_functions(M) + M - 1) / M; }
+
 enum StatusBits : int { ST_NONFINITE = 1, ST_ZERO_DENOM = 2, ST_TIMEOUT = 4 };
 
 // A tile: up to TILE consecutive points of one (atom, image) segment in GPU point order.
@@ -92,9 +101,14 @@ struct View {
     const unsigned char* pt_first;   // [S] 1 if no tile of an earlier apply colour covers this grid point
     double2* gauge_d;      // [S] (cos, sin) of A.d_j, d_j = point minus atom centre (Sec. V, Eq. 16)
     float4* gauge_f;       // [S] the same as FP32 pairs (cos_hi, sin_hi, cos_lo, sin_lo)
-    double* phid64;        // [3][sum S_I M_I] orbitals times the displacement component d_a (Eq. 17)
+    // Tables of the current (Eq. 17).  An atom's orbitals are phi_m = f(r) sum_k A_mk q_k(d) with q_k the monomials
+    // of degree l, so the functions phi_m d_a of the three directions lie in the span of f(r) times the monomials
+    // of degree l + 1: 3, 6, 10, 15 functions for l = 0..3 instead of 3 (2l + 1).  Table t holds functions t M ..
+    // t M + M - 1 in the layout of phi64 (zeros past the last one); an atom has cur_tables(M) of them.
+    double* phid64;        // [3][sum S_I M_I]
     float* phid_hi;        // [3][sum S_I M_I] FP32 split of phid64
     float* phid_lo;
+    double* cur_A;         // [natoms][MAXM][CUR_MAXQ] A_mk
     double* phi64;         // [sum S_I M_I]
     float* phi_hi;
     float* phi_lo;
@@ -174,7 +188,7 @@ struct Ctx {
     double* d_coef_one = nullptr;
     double* d_taylor = nullptr;      // [MAX_TAYLOR] complex Taylor coefficients -i dt / j
     double* d_forces = nullptr;      // [natoms][3]
-    double* d_current = nullptr;     // [natoms][3] per-atom Hubbard current
+    double* d_current = nullptr;     // [natoms][CUR_SPLIT][3] partial sums of the per-atom Hubbard current
     double* d_fll = nullptr;         // [natoms][2] E_ee, E_DC of App. A
     int* d_sink = nullptr;           // [1] output of the access-ceiling pass
     std::vector<int> h_coul_set;     // host copies, so hot-path calls never read the device
@@ -250,14 +264,16 @@ cudaError_t launch_coefvec_batch(const BatchLaunch& b, cudaStream_t st);
 // Taylor step in the span of the orbitals: cv = sum_{j=1}^{order} c_j V p_{j-1}, p_0 = p, p_j = c_j O V p_{j-1}
 // (O: the block overlap above), coefs = the order complex c_j on the device.
 cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double* coefs, bool gauge, cudaStream_t st);
-// Projections onto three orbital tables (v.phi* + a * v.phi_dir_stride, a = 0..2) in one launch, the
-// directions interleaved per tile so that the three reads of a tile's states share L2; results go to
-// p_out + a * p_stride.
+// Projections onto the tables of the current (v.phi* + t * v.phi_dir_stride) in one launch, interleaved per tile so
+// that the reads of a tile's states share L2; results go to p_out + t * p_stride.
 cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, dftu_f64_mode mode, int nbands,
                                 int64_t sk, int64_t ss, int64_t sn, bool gauge, double2* p_out, int64_t p_stride,
                                 cudaStream_t st);
-cudaError_t launch_displaced_orbitals(const View& v, int64_t phi_total, cudaStream_t st);
-cudaError_t launch_current(const View& v, const double* f, int nbands, double* Jat, cudaStream_t st);
+// The tables of the current; T: the atoms' Loewdin matrices left by launch_lowdin.
+cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, const double* radial_tab, const int* radial_off,
+                                  const int* radial_nr, const double* radial_dr, cudaStream_t st);
+// Jpart[atom][CUR_SPLIT][3]: partial sums of the per-atom current, to be added in order.
+cudaError_t launch_current(const View& v, const double* f, int nbands, double* Jpart, cudaStream_t st);
 cudaError_t launch_taylor_coefs(double dt, int order, double* coefs, cudaStream_t st);
 cudaError_t launch_forces(const View& v, const double* f, int nbands, double* F, cudaStream_t st);
 cudaError_t launch_fll(const View& v, double* out, cudaStream_t st);

@@ -118,6 +118,11 @@ __device__ __forceinline__ void reduce_item(const View& v, int nbands, int64_t i
 
 __global__ void __launch_bounds__(CTA, 2) k_tile_reduce(View v, int nbands) { reduce_item(v, nbands, blockIdx.x, 0, 0); }
 
+// The tables of the current (blockIdx.y) in one launch, each into its slice of p.
+__global__ void __launch_bounds__(CTA, 2) k_tile_reduce_tables(View v, int nbands, int64_t p_stride) {
+    if ((int)blockIdx.y < cur_tables(v.atom_M[blockIdx.x % v.natoms])) reduce_item(v, nbands, blockIdx.x, blockIdx.y, p_stride);
+}
+
 __global__ void __launch_bounds__(CTA, 2) k_tile_reduce_batch(const View* __restrict__ views, const ProjArgs* __restrict__ args) {
     reduce_item(views[blockIdx.y], args[blockIdx.y].nbands, blockIdx.x, 0, 0);
 }
@@ -197,14 +202,10 @@ cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, 
     else if (mode == DFTU_F64_NATIVE) e = gauge ? run_project<P_F64, 8, 1, 4, 0, 2, 1, 3>(v, a, st) : run_project<P_F64, 8, 1, 4, 0, 2, 0, 3>(v, a, st);
     else e = gauge ? run_project<P_PAIR, 8, 8, 8, 5, 2, 1, 3>(v, a, st) : run_project<P_PAIR, 8, 8, 8, 5, 2, 0, 3>(v, a, st);
     if (e != cudaSuccess) return e;
-    for (int d = 0; d < 3; ++d) {
-        View vd = v;
-        vd.part = v.part + d * v.part_dir_stride;
-        vd.p = p_out + d * p_stride;
-        e = launch_tile_reduce(vd, nbands, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    View vd = v;
+    vd.p = p_out;
+    k_tile_reduce_tables<<<dim3((unsigned)reduce_ctas(v, nbands), 3), CTA, 0, st>>>(vd, nbands, p_stride);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_project_batch(const BatchLaunch& b, dftu_prec prec, dftu_f64_mode mode, int variant, cudaStream_t st) {

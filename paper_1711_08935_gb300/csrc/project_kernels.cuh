@@ -713,7 +713,7 @@ __device__ __forceinline__ void project_item(const View& v, const ProjArgs& a, i
     }
 }
 
-// NDIR > 1: blockIdx.x = tile * NDIR + direction, so the CTAs of one tile and band chunk for the
+// NDIR > 1: blockIdx.x = tile * NDIR + table, so the CTAs of one tile and band chunk for the
 // NDIR orbital tables are neighbours in the launch and read the same states while they sit in L2.
 template <int POL, int Q, int CH, int NBG, int PF, int MINB, int G, int NDIR = 1, int NT = CTA, int TP = TILE>
 __global__ void __launch_bounds__(NT, MINB) k_project(View v, ProjArgs a, int nbg) {
@@ -721,6 +721,7 @@ __global__ void __launch_bounds__(NT, MINB) k_project(View v, ProjArgs a, int nb
     __shared__ int s_pe;
     const int tile = (NDIR == 1) ? (int)blockIdx.x : (int)blockIdx.x / NDIR;
     const int dir = (NDIR == 1) ? 0 : (int)blockIdx.x % NDIR;
+    if (NDIR > 1 && dir >= cur_tables(v.tiles[tile].M)) return;   // the atom has fewer tables
     project_item<POL, Q, CH, NBG, PF, G, NT, TP>(v, a, tile, blockIdx.z, blockIdx.y, nbg, smem, &s_pe, dir);
 }
 

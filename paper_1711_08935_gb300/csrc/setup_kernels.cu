@@ -138,6 +138,92 @@ cudaError_t launch_orbitals(const View& v, const double* radial_tab, const int* 
     return cudaGetLastError();
 }
 
+// Coefficients of real_ylm times r^l on the monomials of degree l (numbered as cur_functions says), row m.
+__device__ void ylm_monomials(int l, double (&c)[MAXM][CUR_MAXQ]) {
+    const double pi = 3.14159265358979323846;
+    for (int m = 0; m < MAXM; ++m)
+        for (int q = 0; q < CUR_MAXQ; ++q) c[m][q] = 0.0;
+    if (l == 0) {
+        c[0][0] = 0.5 / sqrt(pi);
+    } else if (l == 1) {   // x, y, z
+        c[0][1] = c[1][2] = c[2][0] = sqrt(3.0 / (4 * pi));
+    } else if (l == 2) {   // xx, xy, xz, yy, yz, zz
+        const double c1 = sqrt(15.0 / (4 * pi)), c2 = sqrt(5.0 / (16 * pi)), c3 = sqrt(15.0 / (16 * pi));
+        c[0][1] = c1; c[1][4] = c1; c[3][2] = c1;
+        c[2][5] = 2 * c2; c[2][0] = c[2][3] = -c2;
+        c[4][0] = c3; c[4][3] = -c3;
+    } else {               // xxx, xxy, xxz, xyy, xyz, xzz, yyy, yyz, yzz, zzz
+        const double c0 = sqrt(35.0 / (32 * pi)), c1 = sqrt(105.0 / (4 * pi)), c2 = sqrt(21.0 / (32 * pi)), c3 = sqrt(7.0 / (16 * pi)),
+                     c5 = sqrt(105.0 / (16 * pi));
+        c[0][1] = 3 * c0; c[0][6] = -c0;
+        c[1][4] = c1;
+        c[2][8] = 4 * c2; c[2][1] = c[2][6] = -c2;
+        c[3][9] = 2 * c3; c[3][2] = c[3][7] = -3 * c3;
+        c[4][5] = 4 * c2; c[4][0] = c[4][3] = -c2;
+        c[5][2] = c5; c[5][7] = -c5;
+        c[6][0] = c0; c[6][3] = -3 * c0;
+    }
+}
+
+// A_mk of every atom: phi_m = sum_m' R Y_m' T_m'm = (R / r^l) sum_k A_mk q_k.  One thread per atom.
+__global__ void k_current_A(View v, const double* __restrict__ T) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= v.natoms) return;
+    const int M = v.atom_M[a];
+    double c[MAXM][CUR_MAXQ];
+    ylm_monomials((M - 1) / 2, c);
+    for (int m = 0; m < M; ++m)
+        for (int q = 0; q < CUR_MAXQ; ++q) {
+            double s = 0.0;
+            for (int mp = 0; mp < M; ++mp) s += c[mp][q] * T[a * MAXM * MAXM + mp * M + m];
+            v.cur_A[((int64_t)a * MAXM + m) * CUR_MAXQ + q] = s;
+        }
+}
+
+// phid[table][point][m] = R / r^l times the monomial of degree l + 1 numbered table M + m, with its FP32 split.
+__global__ void k_current_tables(View v, int64_t phi_total, const double* __restrict__ rtab, const int* __restrict__ roff,
+                                 const int* __restrict__ rnr, const double* __restrict__ rdr) {
+    const Tile t = v.tiles[blockIdx.x];
+    const int i = threadIdx.x;
+    if (i >= t.np) return;
+    const int64_t j = t.p0 + i;
+    const int a = t.atom, sp = v.atom_species[a], M = t.M, l = (M - 1) / 2;
+    const int ix = v.pt_u[3 * j], jy = v.pt_u[3 * j + 1], kz = v.pt_u[3 * j + 2];
+    const double dx = __dsub_rn(__dadd_rn(__dmul_rn((double)ix, v.h0), v.o0), v.atom_pos[3 * a]);
+    const double dy = __dsub_rn(__dadd_rn(__dmul_rn((double)jy, v.h1), v.o1), v.atom_pos[3 * a + 1]);
+    const double dz = __dsub_rn(__dadd_rn(__dmul_rn((double)kz, v.h2), v.o2), v.atom_pos[3 * a + 2]);
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    const double r = sqrt(d2);
+    double g = radial_interp(rtab + roff[sp], rnr[sp], rdr[sp], r);
+    if (l > 0) g = r == 0.0 ? 0.0 : (l == 1 ? g / r : l == 2 ? g / d2 : g / (d2 * r));
+    const int64_t e0 = t.phi0 + (int64_t)i * M;
+    const int nf = cur_functions(M);
+    for (int fn = 0; fn < cur_tables(M) * M; ++fn) {
+        double y = 0.0;
+        if (fn < nf) {
+            int tt = 0;
+            while ((tt + 1) * (tt + 2) / 2 <= fn) ++tt;
+            const int k = fn - tt * (tt + 1) / 2;
+            y = g;
+            for (int q = 0; q < l + 1 - tt; ++q) y *= dx;
+            for (int q = 0; q < tt - k; ++q) y *= dy;
+            for (int q = 0; q < k; ++q) y *= dz;
+        }
+        const int64_t o = (fn / M) * phi_total + e0 + fn % M;
+        const float hi = __double2float_rn(y);
+        v.phid64[o] = y;
+        v.phid_hi[o] = hi;
+        v.phid_lo[o] = __double2float_rn(y - (double)hi);
+    }
+}
+
+cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, const double* radial_tab, const int* radial_off,
+                                  const int* radial_nr, const double* radial_dr, cudaStream_t st) {
+    k_current_A<<<(v.natoms + 63) / 64, 64, 0, st>>>(v, T);
+    k_current_tables<<<v.ntiles, TILE, 0, st>>>(v, phi_total, radial_tab, radial_off, radial_nr, radial_dr);
+    return cudaGetLastError();
+}
+
 // S_{mm'} = dV sum_j phi_m phi_m' over the atom's points; one CTA per (atom, m m'), fixed-order tree reduction.
 // (All 25 sums of a d shell in one CTA, one after the other: 818 us for 16 atoms of 24405 and 11513 points, a
 // serial chain on 16 SMs; 60 us with a CTA each.)
