@@ -591,8 +591,9 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
     if (!smem_configured((const void*)fn, (int)smem)) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // A colour with few tiles (where spheres overlap) or a small call leaves SMs idle with NBG groups of bands per
-    // CTA, and is then one chain of latencies: it takes one group of 32 lanes per band.  The update of a point
-    // does not depend on the shape.
+    // CTA, and is then one chain of latencies: below half the GPU's slots it takes one group of 32 lanes per band (one
+    // tile, 256 complex64 bands: 34 -> 13 us; 79 tiles, 316 of 456 slots, would slow down: 63 -> 70).  The update of
+    // a point does not depend on the shape.
     auto small = k_apply<POL, 32, 1, 4, PF, G>;
     if (!smem_configured((const void*)small, (int)smem)) e = cudaFuncSetAttribute(small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -602,7 +603,7 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
         if (n == 0) continue;
         a.tile_list = color_order + color_beg[c];
         dim3 grid(n, (a.nbands + BPC * NBG - 1) / (BPC * NBG), v.nk * v.ns);
-        if ((int64_t)grid.x * grid.y * grid.z >= slots) fn<<<grid, CTA, smem, st>>>(v, a);
+        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) fn<<<grid, CTA, smem, st>>>(v, a);
         else small<<<dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st>>>(v, a);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
