@@ -735,13 +735,14 @@ static cudaError_t run_apply_batch(const BatchLaunch& b, const double* coef, int
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CTA, smem);
     if (e != cudaSuccess) return e;
-    for (size_t c = 0; c + 1 < b.color_beg.size(); ++c) {
+    const size_t ncol = b.color_beg.size() - 1;
+    e = cudaMemsetAsync(b.counter, 0, std::max<size_t>(1, ncol) * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    for (size_t c = 0; c < ncol; ++c) {
         int n = b.color_beg[c + 1] - b.color_beg[c];
         if (n == 0) continue;
-        e = cudaMemsetAsync(b.counter, 0, sizeof(int), st);
-        if (e != cudaSuccess) return e;
         int grid = std::max(1, std::min(per_sm * nsm, n));
-        fn<<<grid, CTA, smem, st>>>(b.views, b.args, b.color_items + b.color_beg[c], n, b.counter, coef, accumulate);
+        fn<<<grid, CTA, smem, st>>>(b.views, b.args, b.color_items + b.color_beg[c], n, b.counter + c, coef, accumulate);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -72,9 +72,14 @@ dftu_status dftu_batch_create(dftu_batch* out, int nsys, const dftu_handle* syst
     L.maxM = 1;
     L.max_atoms = 1;
     L.max_ns = 1;
-    for (int s = 0; s < nsys; ++s) {
+    for (auto* c : b->members) views.push_back(c->v);
+    // The persistent kernels take items in this order; a system's items all take its whole band count, so the systems
+    // with the most bands come first and the short items fill the end of the launch.
+    std::vector<int> order(nsys);
+    for (int s = 0; s < nsys; ++s) order[s] = s;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->members[x]->max_bands > b->members[y]->max_bands; });
+    for (int s : order) {
         Ctx* c = b->members[s];
-        views.push_back(c->v);
         L.maxM = std::max(L.maxM, c->v.maxM);
         L.max_atoms = std::max(L.max_atoms, (int)c->atoms.size());
         L.max_ns = std::max(L.max_ns, c->spin == DFTU_NONCOLLINEAR ? 1 : c->ns);
@@ -98,7 +103,8 @@ dftu_status dftu_batch_create(dftu_batch* out, int nsys, const dftu_handle* syst
     if (e == cudaSuccess) e = cudaMalloc(&b->d_color_items, std::max<size_t>(1, citems.size()) * sizeof(int4));
     if (e == cudaSuccess && !citems.empty())
         e = cudaMemcpy(b->d_color_items, citems.data(), citems.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int));
+    // one queue counter per launch of an apply (its colours), so that one memset serves them all
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, std::max<size_t>(1, (size_t)ncol) * sizeof(int));
     if (prev >= 0) cudaSetDevice(prev);
     if (e != cudaSuccess) {
         cudaFree(b->d_views); cudaFree(b->d_items); cudaFree(b->d_color_items); cudaFree(b->d_counter);

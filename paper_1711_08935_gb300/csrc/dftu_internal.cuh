@@ -212,7 +212,7 @@ struct BatchLaunch {
     int nitems;
     const int4* color_items;  // work items of the apply, grouped by colour
     std::vector<int> color_beg;
-    int* counter;             // work-queue counter (reset before each persistent launch)
+    int* counter;             // work-queue counters, one per apply colour (reset before the launches that use them)
     int nsys;
     int maxM;
     int64_t max_reduce;       // max over systems of (k*spin rows) * nbands * sum M
