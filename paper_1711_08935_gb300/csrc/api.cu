@@ -858,7 +858,7 @@ dftu_status dftu_taylor_step(dftu_handle h, void* psi, void* work, dftu_prec pre
     if (e == cudaSuccess) e = launch_acbn0(c->v, st);
     if (e == cudaSuccess) e = launch_taylor_coefs(dt, order, c->d_taylor, st);
     // the terms' coefficients in the span of the orbitals, then one scatter of their sum onto psi
-    if (e == cudaSuccess) e = launch_taylor_cv(c->v, nbands, order, c->d_taylor, G, st);
+    if (e == cudaSuccess) e = launch_taylor_cv(c->v, nbands, order, c->d_taylor, G, true, st);
     if (e == cudaSuccess)
         e = launch_apply(c->v, psi, prec, c->f64_mode, nbands, sk, ss, sn, c->d_coef_one, c->d_color_order, c->color_beg, va, 1, st, G);
     if (e != cudaSuccess) return cuda_fail(c, e, "taylor_step");
@@ -900,7 +900,7 @@ dftu_status dftu_taylor_steps(dftu_handle h, void* psi, dftu_prec prec, int nban
         e = launch_nbar(c->v, nbands, st);
         if (e == cudaSuccess) e = launch_occupations(c->v, f, nbands, st);
         if (e == cudaSuccess) e = launch_acbn0(c->v, st);
-        if (e == cudaSuccess) e = launch_taylor_cv(c->v, nbands, order, c->d_taylor, G, st);
+        if (e == cudaSuccess) e = launch_taylor_cv(c->v, nbands, order, c->d_taylor, G, step == 0, st);
         if (e != cudaSuccess) break;
         if (fused) {
             e = launch_apply_project_c64(c->v, psi, nbands, sk, ss, sn, c->d_coef_one, c->d_color_order, c->color_beg, st);

@@ -456,6 +456,7 @@ __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, in
     int* s_idx = reinterpret_cast<int*>(smem);
     constexpr int BPW = 32 / Q;
     constexpr int BPC = (CTA / 32) * BPW;
+    if (G) dependent_wait();   // the phase table may be the kernel before's
     const Tile t = v.tiles[tile_id];
     const int k = ks / v.ns;
     const int M = t.M;
@@ -511,6 +512,7 @@ __device__ __forceinline__ void apply_item(const View& v, const ApplyArgs& a, in
                 reinterpret_cast<float4*>(s_gauge)[i] = (i < t.np) ? v.gauge_f[t.p0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const int mo = v.atom_moff[t.atom];
+    dependent_wait();   // coefficients and states
     for (int g = 0; g < NBG; ++g) {
         const int band0 = (chunk * NBG + g) * BPC;
         if (band0 >= a.nbands) break;
@@ -603,9 +605,8 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
         if (n == 0) continue;
         a.tile_list = color_order + color_beg[c];
         dim3 grid(n, (a.nbands + BPC * NBG - 1) / (BPC * NBG), v.nk * v.ns);
-        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) fn<<<grid, CTA, smem, st>>>(v, a);
-        else small<<<dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st>>>(v, a);
-        e = cudaGetLastError();
+        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) e = launch_kernel(starts_early(grid), fn, grid, CTA, smem, st, v, a);
+        else e = launch_dependent(small, dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st, v, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -693,7 +694,11 @@ __device__ __forceinline__ void coefvec_elem(const View& v, int nbands, int64_t 
     v.cv[((int64_t)ks * v.max_bands + band) * v.MT + j] = make_double2(re, im);
 }
 
-__global__ void k_coefvec(View v, int nbands) { coefvec_elem(v, nbands, (int64_t)blockIdx.x * blockDim.x + threadIdx.x); }
+__global__ void k_coefvec(View v, int nbands) {
+    dependent_release();
+    dependent_wait();
+    coefvec_elem(v, nbands, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+}
 
 __global__ void k_coefvec_batch(const View* __restrict__ views, const ProjArgs* __restrict__ args) {
     coefvec_elem(views[blockIdx.y], args[blockIdx.y].nbands, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
@@ -701,8 +706,7 @@ __global__ void k_coefvec_batch(const View* __restrict__ views, const ProjArgs* 
 
 cudaError_t launch_coefvec(const View& v, int nbands, cudaStream_t st) {
     const int64_t n = (int64_t)v.nk * v.ns * nbands * v.MT;
-    k_coefvec<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(v, nbands);
-    return cudaGetLastError();
+    return launch_dependent(k_coefvec, (unsigned)((n + 255) / 256), 256, 0, st, v, nbands);
 }
 
 cudaError_t launch_coefvec_batch(const BatchLaunch& b, cudaStream_t st) {

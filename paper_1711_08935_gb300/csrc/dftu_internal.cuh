@@ -263,7 +263,8 @@ cudaError_t launch_access_ceiling(const View& v, void* psi, dftu_prec prec, int 
 cudaError_t launch_coefvec_batch(const BatchLaunch& b, cudaStream_t st);
 // Taylor step in the span of the orbitals: cv = sum_{j=1}^{order} c_j V p_{j-1}, p_0 = p, p_j = c_j O V p_{j-1}
 // (O: the block overlap above), coefs = the order complex c_j on the device.
-cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double* coefs, bool gauge, cudaStream_t st);
+// phases: evaluate the blocks' phases first (the first step of a call; A does not change within one).
+cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double* coefs, bool gauge, bool phases, cudaStream_t st);
 // Projections onto the tables of the current (v.phi* + t * v.phi_dir_stride) in one launch, interleaved per tile so
 // that the reads of a tile's states share L2; results go to p_out + t * p_stride.
 cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, dftu_f64_mode mode, int nbands,
@@ -293,6 +294,41 @@ bool smem_configured(const void* fn, int bytes);
 
 // SMs of the current device (looked up once per device).
 int sm_count();
+
+#ifdef __CUDACC__
+// The kernels of a step run back to back on one stream, many of them for a few microseconds.  Launched dependently, a
+// kernel's blocks start while the last blocks of the one before it still run: they read the handle's constant tables
+// (tiles, grid indices, orbitals), then wait for the kernel before to complete.  Every kernel launched with
+// launch_dependent calls dependent_wait before it reads or writes anything else, and some thread of every grid does,
+// so completion stays in stream order.  Isolated d shell, one step: 94 -> 76 us; small oxide cell: 192 -> 165.
+// The gather and the scatter, whose blocks fill an SM's shared memory, start early only as a small grid and never
+// release the kernel after them early, and the Taylor recursion is launched plainly: an SM keeps its split of shared
+// memory and L1 until it has drained, so blocks that come in beside others' run under theirs as long as the grid lasts
+// (four real-time steps of 64 atoms: 2380 us with all launches plain, 2545 with all dependent, 2363 with this rule).
+__device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependent_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_kernel(bool dependent, void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_kernel(true, fn, grid, threads, smem, st, args...);
+}
+// A gather or scatter grid of at most one wave (two CTAs per SM): its first staging is a visible part of it.
+inline bool starts_early(dim3 grid) { return (int64_t)grid.x * grid.y * grid.z <= 2 * (int64_t)sm_count(); }
+#endif
 
 // Coulomb integrals of one atom's orbitals (blocking); W_out [P][P] with P = M(M+1)/2 pair index.
 int coulomb_atom(const View& v, const Ctx& c, int atom, double* V_dev, std::string& err);

@@ -32,7 +32,11 @@ __device__ __forceinline__ void nbar_warp(const View& v, int nbands, int64_t w) 
     if (lane == 0) v.nbar[((int64_t)row * v.max_bands + band) * v.nspecies + sp] = acc;
 }
 
-__global__ void k_nbar(View v, int nbands) { nbar_warp(v, nbands, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); }
+__global__ void k_nbar(View v, int nbands) {
+    dependent_release();
+    dependent_wait();
+    nbar_warp(v, nbands, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+}
 
 __global__ void k_nbar_batch(const View* __restrict__ views, const ProjArgs* __restrict__ args) {
     nbar_warp(views[blockIdx.y], args[blockIdx.y].nbands, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -115,7 +119,9 @@ __device__ __forceinline__ void occupations_block(const View& v, const double* _
     if (threadIdx.x == 0) v.occ_count[mat] = 0;
 }
 
-__global__ void k_occupations(View v, const double* __restrict__ f, int nbands) {
+__global__ void k_occupations(View v, const double* f, int nbands) {
+    dependent_release();
+    dependent_wait();
     occupations_block(v, f, nbands, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -279,7 +285,11 @@ __device__ __forceinline__ void acbn0_atom(const View& v, int a) {
     }
 }
 
-__global__ void __launch_bounds__(ACB_CTA) k_acbn0(View v) { acbn0_atom(v, blockIdx.x); }
+__global__ void __launch_bounds__(ACB_CTA) k_acbn0(View v) {
+    dependent_release();
+    dependent_wait();
+    acbn0_atom(v, blockIdx.x);
+}
 
 __global__ void __launch_bounds__(ACB_CTA) k_acbn0_batch(const View* __restrict__ views) {
     const View& v = views[blockIdx.y];
@@ -408,19 +418,16 @@ cudaError_t launch_fll(const View& v, double* out, cudaStream_t st) {
 cudaError_t launch_nbar(const View& v, int nbands, cudaStream_t st) {
     int rows = v.noncollinear ? v.nk : v.nk * v.ns;
     int64_t n = (int64_t)rows * nbands * v.nspecies;   // warps, 8 per CTA
-    k_nbar<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(v, nbands);
-    return cudaGetLastError();
+    return launch_dependent(k_nbar, (unsigned)((n + 7) / 8), 256, 0, st, v, nbands);
 }
 
 cudaError_t launch_occupations(const View& v, const double* f, int nbands, cudaStream_t st) {
     dim3 grid(v.natoms, v.noncollinear ? 1 : v.ns, OCC_SPLIT);
-    k_occupations<<<grid, CTA, 0, st>>>(v, f, nbands);
-    return cudaGetLastError();
+    return launch_dependent(k_occupations, grid, CTA, 0, st, v, f, nbands);
 }
 
 cudaError_t launch_acbn0(const View& v, cudaStream_t st) {
-    k_acbn0<<<v.natoms, ACB_CTA, 0, st>>>(v);
-    return cudaGetLastError();
+    return launch_dependent(k_acbn0, v.natoms, ACB_CTA, 0, st, v);
 }
 
 cudaError_t launch_occupations_batch(const BatchLaunch& b, cudaStream_t st) {

@@ -116,7 +116,11 @@ __device__ __forceinline__ void reduce_item(const View& v, int nbands, int64_t i
     }
 }
 
-__global__ void __launch_bounds__(CTA, 2) k_tile_reduce(View v, int nbands) { reduce_item(v, nbands, blockIdx.x, 0, 0); }
+__global__ void __launch_bounds__(CTA, 2) k_tile_reduce(View v, int nbands) {
+    dependent_release();
+    dependent_wait();
+    reduce_item(v, nbands, blockIdx.x, 0, 0);
+}
 
 // The tables of the current (blockIdx.y) in one launch, each into its slice of p.
 __global__ void __launch_bounds__(CTA, 2) k_tile_reduce_tables(View v, int nbands, int64_t p_stride) {
@@ -188,8 +192,7 @@ cudaError_t launch_project_c64_tiles(const View& sub, const void* psi, int nband
 }
 
 cudaError_t launch_tile_reduce(const View& v, int nbands, cudaStream_t st) {
-    k_tile_reduce<<<(unsigned)reduce_ctas(v, nbands), CTA, 0, st>>>(v, nbands);
-    return cudaGetLastError();
+    return launch_dependent(k_tile_reduce, (unsigned)reduce_ctas(v, nbands), CTA, 0, st, v, nbands);
 }
 
 cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, dftu_f64_mode mode, int nbands,

@@ -644,6 +644,7 @@ template <int POL, int Q, int CH, int NBG, int PF, int G, int NT = CTA, int TP =
 __device__ __forceinline__ void project_item(const View& v, const ProjArgs& a, int tile_id, int ks, int chunk, int nbg,
                                              unsigned char* smem, int* s_pe, int dir = 0) {
     int* s_idx = reinterpret_cast<int*>(smem);
+    if (G) dependent_wait();   // the phase table may be the kernel before's
     const Tile t = v.tiles[tile_id];
     const int64_t ph0 = t.phi0 + dir * v.phi_dir_stride;   // this table's rows of the tile
     const int64_t poff = dir * v.part_dir_stride;
@@ -700,6 +701,7 @@ __device__ __forceinline__ void project_item(const View& v, const ProjArgs& a, i
     // (65 complex128 bands are two groups of 32 and one of one band, which used to cost as much as a full one).
     // Only in the default shapes; the split depends on the band count alone, so every launch of a shape sums in
     // the same order.
+    dependent_wait();   // the states
     constexpr bool TAIL = POL == P_PAIR && Q == 8 && CH == 8 && (PF == 5 || PF == 1);   // (the complex64 kernel would spill)
     const int pe = *s_pe;
     const int ng = NBG ? NBG : nbg;
@@ -795,8 +797,7 @@ static cudaError_t run_project(const View& v, const ProjArgs& a, cudaStream_t st
     constexpr int BPC = (NT / 32) * (32 / Q) * LaneBands<POL>::value;
     const int nbg = BAL ? balanced_groups(NBG, BPC, a.nbands, (int64_t)vl.ntiles * NDIR * vl.nk * vl.ns, MINB * sm_count()) : NBG;
     dim3 grid(vl.ntiles * NDIR, (a.nbands + BPC * nbg - 1) / (BPC * nbg), vl.nk * vl.ns);
-    fn<<<grid, NT, smem, st>>>(vl, a, nbg);
-    return cudaGetLastError();
+    return launch_kernel(starts_early(grid), fn, grid, NT, smem, st, vl, a, nbg);
 }
 
 // The default shape of a table row (variant 0): run_project with its thread count and tiling in the last

@@ -18,12 +18,13 @@ namespace dftu {
 
 
 // The default shape, with fewer bands per CTA where the grid would not fill the GPU (balanced_groups).  Calls so
-// small that single groups on the 1024-point tiles leave half the SMs idle are one chain of latencies per CTA: they
+// small that single groups on the 1024-point tiles do not fill the GPU are one chain of latencies per CTA: they
 // run on the 512-point tiles, and with 16 lanes per band while those too leave SMs idle.
-// Isolated d shell, 21 bands (10 CTAs -> 40): 30.3 -> 14.8 us.
+// Isolated d shell, 21 bands (10 CTAs -> 40): 30.3 -> 14.8 us; small oxide cell, 23 bands in 4 (k, spin) (204 CTAs ->
+// 368): 46.9 -> 40.4.
 static cudaError_t project_pair_default(const View& v, const ProjArgs& a, cudaStream_t st, View* used) {
     const int64_t sms = sm_count(), rows = (int64_t)v.nk * v.ns, groups = (a.nbands + 31) / 32;
-    if (v.nptiles * groups * rows >= sms) return run_project_default<DFTU_PROJECT_DEFAULT_PAIR>(v, a, st, used);
+    if (v.nptiles * groups * rows >= 2 * sms) return run_project_default<DFTU_PROJECT_DEFAULT_PAIR>(v, a, st, used);
     if (v.ntiles * groups * rows >= sms) return run_project<P_PAIR, 8, 8, 1, 1, 2, 0, 1, 256, TILE>(v, a, st, used);
     return run_project<P_PAIR, 16, 8, 1, 1, 2, 0, 1, 256, TILE>(v, a, st, used);
 }

@@ -20,6 +20,8 @@ constexpr int TAYLOR_CTA = 512;   // most threads per state
 
 // exp(+i k.D_b), times exp(+i A.Dg_b) when the gauge phases are on, for every (k, block).
 __global__ void k_block_phases(View v, int gauge) {
+    dependent_release();
+    dependent_wait();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= v.nk * v.nblk) return;
     const int k = g / v.nblk, b = g - k * v.nblk;
@@ -139,11 +141,10 @@ __global__ void __launch_bounds__(TAYLOR_CTA) k_taylor_cv(View v, int nbands, in
         }
 }
 
-cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double* coefs, bool gauge, cudaStream_t st) {
-    if (v.nblk > 0) {
+cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double* coefs, bool gauge, bool phases, cudaStream_t st) {
+    if (phases && v.nblk > 0) {
         const int n = v.nk * v.nblk;
-        k_block_phases<<<(n + 127) / 128, 128, 0, st>>>(v, gauge ? 1 : 0);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_dependent(k_block_phases, (n + 127) / 128, 128, 0, st, v, gauge ? 1 : 0);
         if (e != cudaSuccess) return e;
     }
     const int rows = (v.noncollinear ? v.nk : v.nk * v.ns) * nbands;
