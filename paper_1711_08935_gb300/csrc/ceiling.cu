@@ -2,7 +2,8 @@
 // once (the projection's gather), or read and written back unchanged (the apply's read-modify-write),
 // with no arithmetic.  The tiles, grid order and lanes per band are those of the streaming kernels, so
 // the time of one pass bounds what the projection and the apply can reach on this GPU; roofline
-// fractions are quoted against it beside the copy bandwidth.
+// fractions are quoted against it beside the copy bandwidth.  Plain loads: the complex64 projection, whose loads fetch
+// 64-byte blocks instead of whole lines, can run above it.
 #include "dftu_internal.cuh"
 
 namespace dftu {

@@ -25,8 +25,8 @@ __device__ __forceinline__ void displacement(const View& v, int64_t j, int atom,
 
 // exp(+i A.d_j) for every sphere point: FP64 (cos, sin) and the FP32 pair split (hi, hi, lo, lo).  The phase is a
 // product over the axes, so a tile needs one FP64 sine and cosine per grid line it touches on each axis (tables in
-// shared memory) and two complex products per point, instead of a sine and cosine per point: 23.3 us on 171 k
-// points by the FP64 pipe.
+// shared memory) and two complex products per point, instead of a sine and cosine per point, which the FP64 pipe
+// bounds: 171 k points, 23.7 -> 13.4 us.  Now a chain of latencies (48 bytes written per point are 1.2 us of it).
 constexpr int GAUGE_TAB = 256;   // grid lines per axis the tables hold; larger tiles evaluate every point
 __global__ void __launch_bounds__(TILE) k_gauge_phases(View v, const double* __restrict__ A) {
     __shared__ double2 tab[3][GAUGE_TAB];
@@ -84,7 +84,8 @@ cudaError_t launch_gauge_phases(const View& v, const double* A, cudaStream_t st)
 // Im sum_xy V_xy [conj(q_x) p_y - conj(p_x) q_y] for a Hermitian V.  With q^a_x = sum_k A_xk P_(k a), P the projections
 // onto the tables of the current and (k a) the function q_k d_a, the sum is sum_k conj(P_(k a)) u_k with
 // u_k = sum_x A_xk (V p)_x: one pass over a state's projections serves the three directions.  Collinear or
-// unpolarised states.  (One CTA per (atom, direction) over the displaced orbitals took 19.3 us on 16 atoms, 192 states.)
+// unpolarised states.  16 atoms, 192 states: 19.3 -> 12.3 us (before: one CTA per (atom, direction) over the displaced
+// orbitals); latency bounds both, so each atom's states are split over CUR_SPLIT CTAs.
 
 template <int M>
 __device__ __forceinline__ void current_states(const View& v, const double* __restrict__ f, int nbands, int atom, int z,
