@@ -605,7 +605,7 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
         if (n == 0) continue;
         a.tile_list = color_order + color_beg[c];
         dim3 grid(n, (a.nbands + BPC * NBG - 1) / (BPC * NBG), v.nk * v.ns);
-        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) e = launch_kernel(starts_early(grid), fn, grid, CTA, smem, st, v, a);
+        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) e = launch_dependent(fn, grid, CTA, smem, st, v, a);
         else e = launch_dependent(small, dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st, v, a);
         if (e != cudaSuccess) return e;
     }

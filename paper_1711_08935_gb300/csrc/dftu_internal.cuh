@@ -301,15 +301,16 @@ int sm_count();
 // (tiles, grid indices, orbitals), then wait for the kernel before to complete.  Every kernel launched with
 // launch_dependent calls dependent_wait before it reads or writes anything else, and some thread of every grid does,
 // so completion stays in stream order.  Isolated d shell, one step: 94 -> 76 us; small oxide cell: 192 -> 165.
-// The gather and the scatter, whose blocks fill an SM's shared memory, start early only as a small grid and never
-// release the kernel after them early, and the Taylor recursion is launched plainly: an SM keeps its split of shared
-// memory and L1 until it has drained, so blocks that come in beside others' run under theirs as long as the grid lasts
-// (four real-time steps of 64 atoms: 2380 us with all launches plain, 2545 with all dependent, 2363 with this rule).
+// Only grids of one wave (two CTAs per SM) start early, the gather and the scatter, whose blocks fill an SM's shared
+// memory, never release the kernel after them early, and the Taylor recursion is launched plainly: an SM keeps its
+// split of shared memory and L1 until it has drained, so blocks that come in beside others' run under theirs as long as
+// the grid lasts (four real-time steps of 64 atoms: 2380 us with all launches plain, 2545 with all dependent, 2363 with
+// the gather, the scatter and the recursion held back).
 __device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependent_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-cudaError_t launch_kernel(bool dependent, void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -319,15 +320,9 @@ cudaError_t launch_kernel(bool dependent, void (*fn)(P...), dim3 grid, int threa
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = dependent ? 1 : 0;
+    cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= 2 * (int64_t)sm_count() ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
 }
-template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
-    return launch_kernel(true, fn, grid, threads, smem, st, args...);
-}
-// A gather or scatter grid of at most one wave (two CTAs per SM): its first staging is a visible part of it.
-inline bool starts_early(dim3 grid) { return (int64_t)grid.x * grid.y * grid.z <= 2 * (int64_t)sm_count(); }
 #endif
 
 // Coulomb integrals of one atom's orbitals (blocking); W_out [P][P] with P = M(M+1)/2 pair index.

@@ -33,7 +33,7 @@ __device__ __forceinline__ void nbar_warp(const View& v, int nbands, int64_t w) 
 }
 
 __global__ void k_nbar(View v, int nbands) {
-    dependent_release();
+    if (gridDim.x <= 256) dependent_release();   // beside a full grid the next kernel's blocks crowd on a few SMs (4096 oxide states, with U, J: 102 -> 66 us)
     dependent_wait();
     nbar_warp(v, nbands, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
 }

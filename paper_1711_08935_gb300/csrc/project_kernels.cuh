@@ -797,7 +797,7 @@ static cudaError_t run_project(const View& v, const ProjArgs& a, cudaStream_t st
     constexpr int BPC = (NT / 32) * (32 / Q) * LaneBands<POL>::value;
     const int nbg = BAL ? balanced_groups(NBG, BPC, a.nbands, (int64_t)vl.ntiles * NDIR * vl.nk * vl.ns, MINB * sm_count()) : NBG;
     dim3 grid(vl.ntiles * NDIR, (a.nbands + BPC * nbg - 1) / (BPC * nbg), vl.nk * vl.ns);
-    return launch_kernel(starts_early(grid), fn, grid, NT, smem, st, vl, a, nbg);
+    return launch_dependent(fn, grid, NT, smem, st, vl, a, nbg);
 }
 
 // The default shape of a table row (variant 0): run_project with its thread count and tiling in the last
