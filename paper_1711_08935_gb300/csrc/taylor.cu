@@ -44,7 +44,7 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 // One CTA per state (k, spin, band; non-collinear: k, band with both components), one thread per element of its
 // vectors where they fit a CTA.  X = p_{j-1}, W = V p_{j-1} and the sum of the a_j live in shared memory (SH), so a
 // term costs two rounds of short dependent loads; states too large for it keep them in global scratch.  64 atoms
-// (277 orbitals), 256 states, order 4: 63 us with 128 threads per state over global memory (three rounds of
+// (277 orbitals), 256 states, order 4: 63 -> 52 us (before: 128 threads per state over global memory, three rounds of
 // elements per phase, every vector read an L2 latency); its FP64 operations alone take 19.
 template <int SH>
 __global__ void __launch_bounds__(TAYLOR_CTA) k_taylor_cv(View v, int nbands, int order, const double2* __restrict__ coefs,
@@ -150,10 +150,14 @@ cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double*
     const int rows = (v.noncollinear ? v.nk : v.nk * v.ns) * nbands;
     const int64_t slice = (int64_t)v.nk * v.ns * v.max_bands * v.MT;   // one slice of the gradient-projection buffer
     const int nel = (v.noncollinear ? 2 : 1) * v.MT;
-    const int nt = std::min(TAYLOR_CTA, (nel + 31) / 32 * 32);
+    // More than four states per SM fill the FP64 pipe with 128 threads each and their vectors in L2, at less cost per state
+    // (1024 states of 277 orbitals: 157 us against 164 in shared memory with a thread per orbital, 169 there with 128
+    // threads; 256 states: 63 against 52).
+    const bool many = rows > 4 * sm_count();
+    const int nt = std::min(many ? 128 : TAYLOR_CTA, (nel + 31) / 32 * 32);
     const size_t smem = 3 * (size_t)nel * sizeof(double2);
     const double2* cf = reinterpret_cast<const double2*>(coefs);
-    if (smem <= 160 * 1024) {
+    if (!many && smem <= 160 * 1024) {
         cudaError_t e = cudaSuccess;
         if (smem > 48 * 1024 && !smem_configured((const void*)k_taylor_cv<1>, (int)smem))
             e = cudaFuncSetAttribute(k_taylor_cv<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -208,3 +208,27 @@ def test_real_time_overlaps_from_shared_points(case):
     t = torch.from_numpy(psi).cuda()
     h.taylor_step(t, None, torch.from_numpy(f).cuda(), 0.8)
     assert rel(t.cpu().numpy(), ref) < 1e-12
+
+
+@pytest.mark.parametrize("nb", [32, 33])
+def test_wide_calls_are_their_narrow_parts(nb):
+    """Calls wide enough for a reduce with a thread per state and orbital and for a recursion on 128 threads, with whole
+    and with ragged groups of bands: copies of a narrow call's states, the copies empty, step as the narrow call does
+    (which the oracle's step pins above)."""
+    s = _cases.overlapping_three_atoms()
+    copies = 3400 // nb
+    psi = _random_states(s, nb, seed=nb)
+    f = np.random.default_rng(nb).uniform(0.2, 1.0, (s.nk, 1, nb))
+    narrow = torch.from_numpy(psi).cuda()
+    wide = narrow.repeat(1, 1, copies, 1).contiguous()
+    fw = torch.zeros((s.nk, 1, nb * copies), dtype=torch.float64, device="cuda")
+    fw[:, :, :nb] = torch.from_numpy(f).cuda()
+    for t, g in ((narrow, torch.from_numpy(f).cuda()), (wide, fw)):
+        h = dftu.handle_for_system(s, t.shape[2])
+        for I in range(len(s.atoms)):
+            h.set_u(I, 0.4, 0.05)
+        h.taylor_step(t, None, g, 0.8)
+        h.close()
+    for c in (0, copies // 2, copies - 1):
+        part = wide[:, :, c * nb:(c + 1) * nb]
+        assert float((part - narrow).abs().max()) <= 1e-12 * float(narrow.abs().max())
