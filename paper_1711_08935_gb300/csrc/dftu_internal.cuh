@@ -300,7 +300,7 @@ int sm_count();
 // kernel's blocks start while the last blocks of the one before it still run: they read the handle's constant tables
 // (tiles, grid indices, orbitals), then wait for the kernel before to complete.  Every kernel launched with
 // launch_dependent calls dependent_wait before it reads or writes anything else, and some thread of every grid does,
-// so completion stays in stream order.  Isolated d shell, one step: 94 -> 76 us; small oxide cell: 192 -> 165.
+// so completion stays in stream order.  Isolated d shell, one step: 94 -> 74 us; small oxide cell: 192 -> 171.
 // Only grids of one wave (two CTAs per SM) start early, the gather and the scatter, whose blocks fill an SM's shared
 // memory, never release the kernel after them early, and the Taylor recursion is launched plainly: an SM keeps its
 // split of shared memory and L1 until it has drained, so blocks that come in beside others' run under theirs as long as
