@@ -80,16 +80,16 @@ cudaError_t launch_gauge_phases(const View& v, const double* A, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Jpart[atom][z][a] = mult sum over the states of split z of w f 2 Im sum_x conj(q^a_x) (V p)_x, which is
-// Im sum_xy V_xy [conj(q_x) p_y - conj(p_x) q_y] for a Hermitian V.  With q^a_x = sum_k A_xk P_(k a), P the projections
-// onto the tables of the current and (k a) the function q_k d_a, the sum is sum_k conj(P_(k a)) u_k with
-// u_k = sum_x A_xk (V p)_x: one pass over a state's projections serves the three directions.  Collinear or
-// unpolarised states.  16 atoms, 192 states: 19.3 -> 12.3 us (before: one CTA per (atom, direction) over the displaced
+// Jpart[atom][z][a] = mult sum over the states of split z of w f Im sum_x conj(q^a_x) (H p)_x, H = V + V^+, which is
+// Im sum_xy V_xy [conj(q_x) p_y - conj(p_x) q_y] for any V (occupation sums that a caller imports need not be
+// Hermitian).  With q^a_x = sum_k A_xk P_(k a), P the projections onto the tables of the current and (k a) the function
+// q_k d_a, the sum is sum_k conj(P_(k a)) u_k with u_k = sum_x A_xk (H p)_x: one pass over a state's projections
+// serves the three directions.  Collinear or unpolarised states.  16 atoms, 192 states: 19.3 -> 12.3 us (before: one CTA per (atom, direction) over the displaced
 // orbitals); latency bounds both, so each atom's states are split over CUR_SPLIT CTAs.
 
 template <int M>
 __device__ __forceinline__ void current_states(const View& v, const double* __restrict__ f, int nbands, int atom, int z,
-                                               const double2* s_V, const double* s_A, double (&acc)[3]) {
+                                               const double2* s_H, const double* s_A, double (&acc)[3]) {
     constexpr int NQ = cur_monomials(M);
     const int mo = v.atom_moff[atom];
     const int64_t slice = (int64_t)v.nk * v.ns * v.max_bands * v.MT;
@@ -108,9 +108,9 @@ __device__ __forceinline__ void current_states(const View& v, const double* __re
             double2 t = make_double2(0.0, 0.0);
 #pragma unroll
             for (int y = 0; y < M; ++y) {
-                const double2 V = s_V[s * M * M + x * M + y];
-                t.x = fma(V.x, p[y].x, fma(-V.y, p[y].y, t.x));
-                t.y = fma(V.x, p[y].y, fma(V.y, p[y].x, t.y));
+                const double2 H = s_H[s * M * M + x * M + y];
+                t.x = fma(H.x, p[y].x, fma(-H.y, p[y].y, t.x));
+                t.y = fma(H.x, p[y].y, fma(H.y, p[y].x, t.y));
             }
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
@@ -130,7 +130,7 @@ __device__ __forceinline__ void current_states(const View& v, const double* __re
                 const double2 P = v.pgrad[(fn / M) * slice + row + fn % M];
                 im = fma(P.x, u[q].y, fma(-P.y, u[q].x, im));
             }
-            acc[a] += 2.0 * w * im;
+            acc[a] += w * im;
         }
     }
 }
@@ -138,18 +138,23 @@ __device__ __forceinline__ void current_states(const View& v, const double* __re
 __global__ void __launch_bounds__(128) k_current(View v, const double* __restrict__ f, int nbands, double* __restrict__ Jpart) {
     const int atom = blockIdx.x, z = blockIdx.y;
     const int M = v.atom_M[atom];
-    __shared__ double2 s_V[2 * MAXM * MAXM];
+    __shared__ double2 s_H[2 * MAXM * MAXM];
     __shared__ double s_A[MAXM * CUR_MAXQ];
     __shared__ double red[3][4];
-    for (int e = threadIdx.x; e < v.ns * M * M; e += blockDim.x) s_V[e] = v.V[v.atom_mat_off[atom] + e];
+    const double2* V = v.V + v.atom_mat_off[atom];
+    for (int e = threadIdx.x; e < v.ns * M * M; e += blockDim.x) {
+        const int x = e / M % M, y = e % M;
+        const double2 a = V[e], b = V[e - x * M - y + y * M + x];
+        s_H[e] = make_double2(a.x + b.x, a.y - b.y);
+    }
     for (int e = threadIdx.x; e < M * CUR_MAXQ; e += blockDim.x) s_A[e] = v.cur_A[(int64_t)atom * MAXM * CUR_MAXQ + e];
     __syncthreads();
     double acc[3] = {0.0, 0.0, 0.0};
     switch (M) {
-        case 1: current_states<1>(v, f, nbands, atom, z, s_V, s_A, acc); break;
-        case 3: current_states<3>(v, f, nbands, atom, z, s_V, s_A, acc); break;
-        case 5: current_states<5>(v, f, nbands, atom, z, s_V, s_A, acc); break;
-        default: current_states<7>(v, f, nbands, atom, z, s_V, s_A, acc); break;
+        case 1: current_states<1>(v, f, nbands, atom, z, s_H, s_A, acc); break;
+        case 3: current_states<3>(v, f, nbands, atom, z, s_H, s_A, acc); break;
+        case 5: current_states<5>(v, f, nbands, atom, z, s_H, s_A, acc); break;
+        default: current_states<7>(v, f, nbands, atom, z, s_H, s_A, acc); break;
     }
     for (int a = 0; a < 3; ++a) {
         for (int off = 16; off > 0; off >>= 1) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], off);
