@@ -500,7 +500,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = dalloc(c, &v.pgrad, (size_t)3 * rowsP * c->max_bands * MT);
     if (e == cudaSuccess) e = dalloc(c, &c->d_forces, (size_t)3 * natoms);
     if (e == cudaSuccess) e = dalloc(c, &c->d_current, (size_t)3 * CUR_SPLIT * natoms);
-    if (e == cudaSuccess) e = dalloc(c, &v.cur_A, (size_t)natoms * MAXM * CUR_MAXQ);
+    if (e == cudaSuccess) e = dalloc(c, &v.cur_A, (size_t)natoms * CUR_MAXF * 3 * MAXM);
     if (e == cudaSuccess) e = dalloc(c, &c->d_fll, (size_t)2 * natoms);
     if (e == cudaSuccess) e = dalloc(c, &v.gauge_d, (size_t)c->S);
     if (e == cudaSuccess) e = dalloc(c, &v.gauge_f, (size_t)c->S);
@@ -530,7 +530,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = launch_orbitals(v, d_rtab, d_roff, d_rnr, d_rdr, 0);
     double* cond = work + (size_t)natoms * MAXM * MAXM;
     if (e == cudaSuccess) e = launch_lowdin(v, work, cond, 0);
-    if (e == cudaSuccess) e = launch_current_tables(v, phi_off, work, d_rtab, d_roff, d_rnr, d_rdr, 0);
+    if (e == cudaSuccess) e = launch_current_tables(v, phi_off, work, c->d_current, d_rtab, d_roff, d_rnr, d_rdr, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(c, e, "setup_atoms: orbitals");
     // S^(-1/2) exists only for orbitals that are linearly independent on the sphere (Sec. III)

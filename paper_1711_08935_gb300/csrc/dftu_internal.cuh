@@ -34,14 +34,12 @@ constexpr int OCC_MAXP = (2 * MAXM) * (2 * MAXM);   // largest matrix (non-colli
 constexpr double LOWDIN_MIN_RATIO = 1e-10;   // smallest accepted lambda_min / lambda_max of an atom's orbital
                                             // overlap; below it S^(-1/2) is refused (orbitals dependent)
 
-constexpr int CUR_MAXQ = 10;   // monomials of degree l <= 3
+// Functions of the current's tables (View::phid64): harmonics of degree l + 1, then of degree l - 1; an atom's tables
+// hold M of them each.
+constexpr int CUR_MAXF = 14;   // l = 3
 constexpr int CUR_SPLIT = 8;   // CTAs sharing an atom's sum over states of the current
-
-// Monomials of degree D are numbered t(t+1)/2 + k for x^(D-t) y^(t-k) z^k, whatever D: multiplying by x keeps the
-// number, by y or z moves it to the next t.
-__host__ __device__ constexpr int cur_functions(int M) { return ((M - 1) / 2 + 2) * ((M - 1) / 2 + 3) / 2; }   // degree l + 1
-__host__ __device__ constexpr int cur_monomials(int M) { return ((M - 1) / 2 + 1) * ((M - 1) / 2 + 2) / 2; }   // degree l
-__host__ __device__ constexpr int cur_tables(int M) { return (cur_functions(M) + M - 1) / M; }
+__host__ __device__ constexpr int cur_functions(int M) { return M == 1 ? 3 : 2 * M; }
+__host__ __device__ constexpr int cur_tables(int M) { return M == 1 ? 3 : 2; }
 
 enum StatusBits : int { ST_NONFINITE = 1, ST_ZERO_DENOM = 2, ST_TIMEOUT = 4 };
 
@@ -101,14 +99,16 @@ struct View {
     const unsigned char* pt_first;   // [S] 1 if no tile of an earlier apply colour covers this grid point
     double2* gauge_d;      // [S] (cos, sin) of A.d_j, d_j = point minus atom centre (Sec. V, Eq. 16)
     float4* gauge_f;       // [S] the same as FP32 pairs (cos_hi, sin_hi, cos_lo, sin_lo)
-    // Tables of the current (Eq. 17).  An atom's orbitals are phi_m = f(r) sum_k A_mk q_k(d) with q_k the monomials
-    // of degree l, so the functions phi_m d_a of the three directions lie in the span of f(r) times the monomials
-    // of degree l + 1: 3, 6, 10, 15 functions for l = 0..3 instead of 3 (2l + 1).  Table t holds functions t M ..
-    // t M + M - 1 in the layout of phi64 (zeros past the last one); an atom has cur_tables(M) of them.
+    // Tables of the current (Eq. 17).  An atom's orbitals are phi_m = R(r) sum_m' Y_lm' T_m'm, so the functions phi_m d_a
+    // of the three directions lie in the span of R(r) r times the real harmonics of degree l + 1 and l - 1: 3, 6, 10, 14
+    // functions for l = 0..3 instead of 3 (2l + 1).  Table t holds functions t M .. t M + M - 1 in the layout of phi64,
+    // scaled per atom so that the largest value lies just below one: the FP32-pair projection's error follows the power
+    // of two above a tile's largest value.  (Unlike monomials of degree l + 1, which are larger than the phi_m d_a that
+    // their differences form, harmonics keep the projections' error: q^a_m is a contraction of theirs.)
     double* phid64;        // [3][sum S_I M_I]
     float* phid_hi;        // [3][sum S_I M_I] FP32 split of phid64
     float* phid_lo;
-    double* cur_A;         // [natoms][MAXM][CUR_MAXQ] A_mk
+    double* cur_A;         // [natoms][CUR_MAXF][3][MAXM]: phi_m d_a = sum_f A[f][a][m] F_f
     double* phi64;         // [sum S_I M_I]
     float* phi_hi;
     float* phi_lo;
@@ -270,8 +270,8 @@ cudaError_t launch_taylor_cv(const View& v, int nbands, int order, const double*
 cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, dftu_f64_mode mode, int nbands,
                                 int64_t sk, int64_t ss, int64_t sn, bool gauge, double2* p_out, int64_t p_stride,
                                 cudaStream_t st);
-// The tables of the current; T: the atoms' Loewdin matrices left by launch_lowdin.
-cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, const double* radial_tab, const int* radial_off,
+// The tables of the current; T: the atoms' Loewdin matrices left by launch_lowdin; peak: scratch, [natoms].
+cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, double* peak, const double* radial_tab, const int* radial_off,
                                   const int* radial_nr, const double* radial_dr, cudaStream_t st);
 // Jpart[atom][CUR_SPLIT][3]: partial sums of the per-atom current, to be added in order.
 cudaError_t launch_current(const View& v, const double* f, int nbands, double* Jpart, cudaStream_t st);

@@ -9,7 +9,7 @@
 // Eq. (17), the Hubbard contribution to the current, is taken as J = sum w f <psi| -i [r, V_U^A] |psi>
 // (the factor i of the velocity operator restored, since <[r, V]> + c.c. of a Hermitian V vanishes).
 // With q^{(a)}_m = <phi_m d_a exp(-i A.d)|psi>, the projections onto orbitals weighted by the a-th
-// displacement component (formed from the projections onto monomials, View::phid64),
+// displacement component (formed from the projections onto harmonics, View::phid64),
 //   J_a = -i sum w f sum_{mm'} V_{mm'} [conj(q_m) p_m' - conj(p_m) q_m'],
 // a real number; it equals dE_U/dA at fixed states.
 #include "dftu_internal.cuh"
@@ -80,31 +80,34 @@ cudaError_t launch_gauge_phases(const View& v, const double* A, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Jpart[atom][z][a] = mult sum over the states of split z of w f Im sum_x conj(q^a_x) (H p)_x, H = V + V^+, which is
+// Jpart[atom][z][a] = mult sum over the states of split z of w f Im sum_x conj(q^a_x) t_x, t = (V + V^+) p, which is
 // Im sum_xy V_xy [conj(q_x) p_y - conj(p_x) q_y] for any V (occupation sums that a caller imports need not be
-// Hermitian).  With q^a_x = sum_k A_xk P_(k a), P the projections onto the tables of the current and (k a) the function
-// q_k d_a, the sum is sum_k conj(P_(k a)) u_k with u_k = sum_x A_xk (H p)_x: one pass over a state's projections
-// serves the three directions.  Collinear or unpolarised states.  16 atoms, 192 states: 19.3 -> 12.3 us (before: one CTA per (atom, direction) over the displaced
-// orbitals); latency bounds both, so each atom's states are split over CUR_SPLIT CTAs.
+// Hermitian).  With q^a_x = sum_f A[f][a][x] P_f, P the projections onto the tables of the current, it is
+// sum_(f, x) A[f][a][x] Im conj(P_f) t_x: one pass over a state's projections serves the three directions.  Collinear or
+// unpolarised states.
+// An atom's states are split over CUR_SPLIT CTAs, and a CTA takes CUR_STATES states at a time, a lane each; its four
+// warps share the rows of t (through shared memory) and the functions f.  Few states, few warps: the FP64 pipe of one
+// SM quarter, 80 cycles an instruction of a warp, would bound a thread per state.
+constexpr int CUR_STATES = 32, CUR_PARTS = 4;
 
 template <int M>
 __device__ __forceinline__ void current_states(const View& v, const double* __restrict__ f, int nbands, int atom, int z,
-                                               const double2* s_H, const double* s_A, double (&acc)[3]) {
-    constexpr int NQ = cur_monomials(M);
-    const int mo = v.atom_moff[atom];
+                                               const double2* s_H, const double* s_A, double2* s_t, double (&acc)[3]) {
+    constexpr int NF = cur_functions(M);
+    const int lane = threadIdx.x % CUR_STATES, part = threadIdx.x / CUR_STATES;
     const int64_t slice = (int64_t)v.nk * v.ns * v.max_bands * v.MT;
     const int total = v.nk * v.ns * nbands;
-    for (int e = z * blockDim.x + threadIdx.x; e < total; e += CUR_SPLIT * blockDim.x) {
+    for (int e0 = z * CUR_STATES; e0 < total; e0 += CUR_SPLIT * CUR_STATES) {
+        const bool in = e0 + lane < total;
+        const int e = in ? e0 + lane : 0;
         const int ks = e / nbands, band = e % nbands, k = ks / v.ns, s = ks % v.ns;
-        const double w = v.wk[k] * f[(int64_t)ks * nbands + band];
-        const int64_t row = ((int64_t)ks * v.max_bands + band) * v.MT + mo;
-        double2 p[M], u[NQ];
+        const double w = in ? v.wk[k] * f[(int64_t)ks * nbands + band] : 0.0;
+        const int64_t row = ((int64_t)ks * v.max_bands + band) * v.MT + v.atom_moff[atom];
+        double2 p[M];
 #pragma unroll
         for (int x = 0; x < M; ++x) p[x] = v.p[row + x];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) u[q] = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int x = 0; x < M; ++x) {
+        __syncthreads();   // the states before have been read
+        for (int x = part; x < M; x += CUR_PARTS) {
             double2 t = make_double2(0.0, 0.0);
 #pragma unroll
             for (int y = 0; y < M; ++y) {
@@ -112,49 +115,45 @@ __device__ __forceinline__ void current_states(const View& v, const double* __re
                 t.x = fma(H.x, p[y].x, fma(-H.y, p[y].y, t.x));
                 t.y = fma(H.x, p[y].y, fma(H.y, p[y].x, t.y));
             }
+            s_t[x * CUR_STATES + lane] = t;
+        }
+        __syncthreads();
+        double im[3] = {0.0, 0.0, 0.0};
+        for (int q = part; q < NF; q += CUR_PARTS) {
+            const double2 P = v.pgrad[(q / M) * slice + row + q % M];
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const double A = s_A[x * CUR_MAXQ + q];
-                u[q].x = fma(A, t.x, u[q].x);
-                u[q].y = fma(A, t.y, u[q].y);
+            for (int x = 0; x < M; ++x) {
+                const double2 t = s_t[x * CUR_STATES + lane];
+                const double c = fma(P.x, t.y, -P.y * t.x);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) im[a] = fma(s_A[(q * 3 + a) * MAXM + x], c, im[a]);
             }
         }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double im = 0.0;
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                int t = 0;
-                while ((t + 1) * (t + 2) / 2 <= q) ++t;
-                const int fn = a == 0 ? q : q + t + a;   // y: next t, same k; z: next t, next k
-                const double2 P = v.pgrad[(fn / M) * slice + row + fn % M];
-                im = fma(P.x, u[q].y, fma(-P.y, u[q].x, im));
-            }
-            acc[a] += w * im;
-        }
+        if (in)   // (a state of weight zero may hold anything)
+            for (int a = 0; a < 3; ++a) acc[a] = fma(w, im[a], acc[a]);
     }
 }
 
-__global__ void __launch_bounds__(128) k_current(View v, const double* __restrict__ f, int nbands, double* __restrict__ Jpart) {
+__global__ void __launch_bounds__(CUR_STATES * CUR_PARTS) k_current(View v, const double* __restrict__ f, int nbands, double* __restrict__ Jpart) {
     const int atom = blockIdx.x, z = blockIdx.y;
     const int M = v.atom_M[atom];
-    __shared__ double2 s_H[2 * MAXM * MAXM];
-    __shared__ double s_A[MAXM * CUR_MAXQ];
-    __shared__ double red[3][4];
+    __shared__ double2 s_H[2 * MAXM * MAXM], s_t[MAXM * CUR_STATES];
+    __shared__ double s_A[CUR_MAXF * 3 * MAXM];
+    __shared__ double red[3][CUR_PARTS];
     const double2* V = v.V + v.atom_mat_off[atom];
     for (int e = threadIdx.x; e < v.ns * M * M; e += blockDim.x) {
         const int x = e / M % M, y = e % M;
         const double2 a = V[e], b = V[e - x * M - y + y * M + x];
         s_H[e] = make_double2(a.x + b.x, a.y - b.y);
     }
-    for (int e = threadIdx.x; e < M * CUR_MAXQ; e += blockDim.x) s_A[e] = v.cur_A[(int64_t)atom * MAXM * CUR_MAXQ + e];
+    for (int e = threadIdx.x; e < CUR_MAXF * 3 * MAXM; e += blockDim.x) s_A[e] = v.cur_A[(int64_t)atom * CUR_MAXF * 3 * MAXM + e];
     __syncthreads();
     double acc[3] = {0.0, 0.0, 0.0};
     switch (M) {
-        case 1: current_states<1>(v, f, nbands, atom, z, s_H, s_A, acc); break;
-        case 3: current_states<3>(v, f, nbands, atom, z, s_H, s_A, acc); break;
-        case 5: current_states<5>(v, f, nbands, atom, z, s_H, s_A, acc); break;
-        default: current_states<7>(v, f, nbands, atom, z, s_H, s_A, acc); break;
+        case 1: current_states<1>(v, f, nbands, atom, z, s_H, s_A, s_t, acc); break;
+        case 3: current_states<3>(v, f, nbands, atom, z, s_H, s_A, s_t, acc); break;
+        case 5: current_states<5>(v, f, nbands, atom, z, s_H, s_A, s_t, acc); break;
+        default: current_states<7>(v, f, nbands, atom, z, s_H, s_A, s_t, acc); break;
     }
     for (int a = 0; a < 3; ++a) {
         for (int off = 16; off > 0; off >>= 1) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], off);
@@ -168,7 +167,7 @@ __global__ void __launch_bounds__(128) k_current(View v, const double* __restric
 }
 
 cudaError_t launch_current(const View& v, const double* f, int nbands, double* Jpart, cudaStream_t st) {
-    k_current<<<dim3(v.natoms, CUR_SPLIT), 128, 0, st>>>(v, f, nbands, Jpart);
+    k_current<<<dim3(v.natoms, CUR_SPLIT), CUR_STATES * CUR_PARTS, 0, st>>>(v, f, nbands, Jpart);
     return cudaGetLastError();
 }
 

@@ -69,7 +69,7 @@ cudaError_t launch_seg_phases(const View& v, cudaStream_t st) {
 }
 
 // Real spherical harmonics, m = -l..l (s: 1 | p: y,z,x | d: xy,yz,3z^2-r^2,xz,x^2-y^2 | f: ...).
-__device__ void real_ylm(int l, double x, double y, double z, double r, double* Y) {
+__host__ __device__ void real_ylm(int l, double x, double y, double z, double r, double* Y) {
     const double pi = 3.14159265358979323846;
     if (l == 0) { Y[0] = 0.5 / sqrt(pi); return; }
     if (r == 0.0) { for (int m = 0; m < 2 * l + 1; ++m) Y[m] = 0.0; return; }
@@ -138,89 +138,164 @@ cudaError_t launch_orbitals(const View& v, const double* radial_tab, const int* 
     return cudaGetLastError();
 }
 
-// Coefficients of real_ylm times r^l on the monomials of degree l (numbered as cur_functions says), row m.
-__device__ void ylm_monomials(int l, double (&c)[MAXM][CUR_MAXQ]) {
-    const double pi = 3.14159265358979323846;
-    for (int m = 0; m < MAXM; ++m)
-        for (int q = 0; q < CUR_MAXQ; ++q) c[m][q] = 0.0;
-    if (l == 0) {
-        c[0][0] = 0.5 / sqrt(pi);
-    } else if (l == 1) {   // x, y, z
-        c[0][1] = c[1][2] = c[2][0] = sqrt(3.0 / (4 * pi));
-    } else if (l == 2) {   // xx, xy, xz, yy, yz, zz
-        const double c1 = sqrt(15.0 / (4 * pi)), c2 = sqrt(5.0 / (16 * pi)), c3 = sqrt(15.0 / (16 * pi));
-        c[0][1] = c1; c[1][4] = c1; c[3][2] = c1;
-        c[2][5] = 2 * c2; c[2][0] = c[2][3] = -c2;
-        c[4][0] = c3; c[4][3] = -c3;
-    } else {               // xxx, xxy, xxz, xyy, xyz, xzz, yyy, yyz, yzz, zzz
-        const double c0 = sqrt(35.0 / (32 * pi)), c1 = sqrt(105.0 / (4 * pi)), c2 = sqrt(21.0 / (32 * pi)), c3 = sqrt(7.0 / (16 * pi)),
-                     c5 = sqrt(105.0 / (16 * pi));
-        c[0][1] = 3 * c0; c[0][6] = -c0;
-        c[1][4] = c1;
-        c[2][8] = 4 * c2; c[2][1] = c[2][6] = -c2;
-        c[3][9] = 2 * c3; c[3][2] = c[3][7] = -3 * c3;
-        c[4][5] = 4 * c2; c[4][0] = c[4][3] = -c2;
-        c[5][2] = c5; c[5][7] = -c5;
-        c[6][0] = c0; c[6][3] = -3 * c0;
+// Real harmonics of degree L on the unit vector (x, y, z), m = -L..L, by the recurrence of the fully normalised
+// Legendre functions over the degree, times Re and Im of (x + i y)^m.  L at compile time: the recurrence's square
+// roots and quotients are then constants.
+template <int L>
+__host__ __device__ __forceinline__ void unit_harmonics(double x, double y, double z, double* Y) {
+    double top = 0.28209479177387814, c = 1.0, s = 0.0;   // sqrt(1 / 4 pi)
+#pragma unroll
+    for (int m = 0; m <= L; ++m) {
+        if (m > 0) {
+            top *= sqrt((2.0 * m + 1.0) / (2.0 * m));
+            const double cx = c * x - s * y;
+            s = c * y + s * x;
+            c = cx;
+        }
+        double p0 = 0.0, p = top;
+#pragma unroll
+        for (int l = m + 1; l <= L; ++l) {
+            const double d = l - 1.0;
+            const double q = sqrt((4.0 * l * l - 1.0) / ((double)l * l - (double)m * m)) *
+                             (z * p - (l == m + 1 ? 0.0 : sqrt((d * d - (double)m * m) / (4.0 * d * d - 1.0)) * p0));
+            p0 = p;
+            p = q;
+        }
+        if (m == 0) Y[L] = p;
+        else { Y[L + m] = 1.4142135623730951 * p * c; Y[L - m] = 1.4142135623730951 * p * s; }
     }
 }
 
-// A_mk of every atom: phi_m = sum_m' R Y_m' T_m'm = (R / r^l) sum_k A_mk q_k.  One thread per atom.
-__global__ void k_current_A(View v, const double* __restrict__ T) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= v.natoms) return;
-    const int M = v.atom_M[a];
-    double c[MAXM][CUR_MAXQ];
-    ylm_monomials((M - 1) / 2, c);
-    for (int m = 0; m < M; ++m)
-        for (int q = 0; q < CUR_MAXQ; ++q) {
+// The harmonics of degree l + 1 and l - 1 that carry n_a Y_lm, 2 M = 4l + 2 of them (l = 0: three).
+template <int l>
+__host__ __device__ __forceinline__ void neighbour_harmonics(double x, double y, double z, double* F) {
+    unit_harmonics<l + 1>(x, y, z, F);
+    if constexpr (l > 0) unit_harmonics<l - 1>(x, y, z, F + 2 * l + 3);
+}
+
+// n_a Y_lm = sum_f c[a][m][f] Y_f over the harmonics f of degree l + 1 (first) and l - 1.
+struct CurCoupling { double c[3][MAXM][CUR_MAXF]; };
+
+// The integrals of n_a Y_lm Y_f over the sphere, by six Gauss-Legendre points in z and twelve angles (exact to degree
+// 11; the products have degree 2l + 2 <= 8).
+template <int l>
+static CurCoupling current_coupling() {
+    constexpr int NZ = 6, NP = 12;
+    const double pi = 3.14159265358979323846;
+    CurCoupling out{};
+    for (int i = 0; i < NZ; ++i) {
+        double z = cos(pi * (i + 0.75) / (NZ + 0.5)), dp = 0.0;   // a root of P_6 by Newton's method
+        for (int it = 0; it < 20; ++it) {
+            double p0 = 1.0, p1 = z;
+            for (int n = 2; n <= NZ; ++n) {
+                const double p2 = ((2 * n - 1) * z * p1 - (n - 1) * p0) / n;
+                p0 = p1;
+                p1 = p2;
+            }
+            dp = NZ * (z * p1 - p0) / (z * z - 1.0);
+            z -= p1 / dp;
+        }
+        const double w = 2.0 / ((1.0 - z * z) * dp * dp) * 2.0 * pi / NP, s = sqrt(1.0 - z * z);
+        for (int q = 0; q < NP; ++q) {
+            const double n[3] = {s * cos(2.0 * pi * q / NP), s * sin(2.0 * pi * q / NP), z};
+            double Y[MAXM], F[CUR_MAXF];
+            real_ylm(l, n[0], n[1], n[2], 1.0, Y);
+            neighbour_harmonics<l>(n[0], n[1], n[2], F);
+            for (int a = 0; a < 3; ++a)
+                for (int m = 0; m < 2 * l + 1; ++m)
+                    for (int f = 0; f < cur_functions(2 * l + 1); ++f) out.c[a][m][f] += w * n[a] * Y[m] * F[f];
+        }
+    }
+    return out;
+}
+
+__device__ __forceinline__ double current_scale(double peak) { return peak > 0.0 ? (1.0 - 0x1p-20) / peak : 1.0; }
+
+// A[f][a][m] of every atom of degree l: phi_m d_a = sum_f A[f][a][m] F_f.  One thread per (atom, f).
+__global__ void k_current_A(View v, int l, CurCoupling C, const double* __restrict__ T, const double* __restrict__ peak) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int a = g / CUR_MAXF, f = g % CUR_MAXF, M = 2 * l + 1;
+    if (a >= v.natoms || v.atom_M[a] != M || f >= cur_functions(M)) return;
+    const double un = 1.0 / current_scale(peak[a]);
+    for (int d = 0; d < 3; ++d)
+        for (int m = 0; m < M; ++m) {
             double s = 0.0;
-            for (int mp = 0; mp < M; ++mp) s += c[mp][q] * T[a * MAXM * MAXM + mp * M + m];
-            v.cur_A[((int64_t)a * MAXM + m) * CUR_MAXQ + q] = s;
+            for (int mp = 0; mp < M; ++mp) s += C.c[d][mp][f] * T[a * MAXM * MAXM + mp * M + m];
+            v.cur_A[(((int64_t)a * CUR_MAXF + f) * 3 + d) * MAXM + m] = s * un;
         }
 }
 
-// phid[table][point][m] = R / r^l times the monomial of degree l + 1 numbered table M + m, with its FP32 split.
-__global__ void k_current_tables(View v, int64_t phi_total, const double* __restrict__ rtab, const int* __restrict__ roff,
-                                 const int* __restrict__ rnr, const double* __restrict__ rdr) {
+// The functions of one point, g times the harmonics; returns the largest magnitude.
+template <int l>
+__device__ __forceinline__ double current_point(const View& v, int64_t phi_total, int64_t phi0, int i, double g, double x, double y, double z) {
+    constexpr int M = 2 * l + 1;
+    double F[cur_functions(M)], m = 0.0;
+    neighbour_harmonics<l>(x, y, z, F);
+#pragma unroll
+    for (int f = 0; f < cur_functions(M); ++f) {
+        const double q = g * F[f];
+        v.phid64[(f / M) * phi_total + phi0 + (int64_t)i * M + f % M] = q;
+        m = fmax(m, fabs(q));
+    }
+    return m;
+}
+
+// phid64[table][point][m] = R r times the harmonic numbered table M + m, and the atom's largest magnitude (its bits
+// order like the numbers; peak starts at zero).
+__global__ void k_current_functions(View v, int64_t phi_total, const double* __restrict__ rtab, const int* __restrict__ roff,
+                                    const int* __restrict__ rnr, const double* __restrict__ rdr, double* __restrict__ peak) {
+    __shared__ unsigned long long top;
+    if (threadIdx.x == 0) top = 0;
+    __syncthreads();
     const Tile t = v.tiles[blockIdx.x];
     const int i = threadIdx.x;
-    if (i >= t.np) return;
-    const int64_t j = t.p0 + i;
-    const int a = t.atom, sp = v.atom_species[a], M = t.M, l = (M - 1) / 2;
-    const int ix = v.pt_u[3 * j], jy = v.pt_u[3 * j + 1], kz = v.pt_u[3 * j + 2];
-    const double dx = __dsub_rn(__dadd_rn(__dmul_rn((double)ix, v.h0), v.o0), v.atom_pos[3 * a]);
-    const double dy = __dsub_rn(__dadd_rn(__dmul_rn((double)jy, v.h1), v.o1), v.atom_pos[3 * a + 1]);
-    const double dz = __dsub_rn(__dadd_rn(__dmul_rn((double)kz, v.h2), v.o2), v.atom_pos[3 * a + 2]);
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    const double r = sqrt(d2);
-    double g = radial_interp(rtab + roff[sp], rnr[sp], rdr[sp], r);
-    if (l > 0) g = r == 0.0 ? 0.0 : (l == 1 ? g / r : l == 2 ? g / d2 : g / (d2 * r));
-    const int64_t e0 = t.phi0 + (int64_t)i * M;
-    const int nf = cur_functions(M);
-    for (int fn = 0; fn < cur_tables(M) * M; ++fn) {
-        double y = 0.0;
-        if (fn < nf) {
-            int tt = 0;
-            while ((tt + 1) * (tt + 2) / 2 <= fn) ++tt;
-            const int k = fn - tt * (tt + 1) / 2;
-            y = g;
-            for (int q = 0; q < l + 1 - tt; ++q) y *= dx;
-            for (int q = 0; q < tt - k; ++q) y *= dy;
-            for (int q = 0; q < k; ++q) y *= dz;
+    if (i < t.np) {
+        const int64_t j = t.p0 + i;
+        const int a = t.atom, sp = v.atom_species[a];
+        const int ix = v.pt_u[3 * j], jy = v.pt_u[3 * j + 1], kz = v.pt_u[3 * j + 2];
+        const double dx = __dsub_rn(__dadd_rn(__dmul_rn((double)ix, v.h0), v.o0), v.atom_pos[3 * a]);
+        const double dy = __dsub_rn(__dadd_rn(__dmul_rn((double)jy, v.h1), v.o1), v.atom_pos[3 * a + 1]);
+        const double dz = __dsub_rn(__dadd_rn(__dmul_rn((double)kz, v.h2), v.o2), v.atom_pos[3 * a + 2]);
+        const double r = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
+        const double g = radial_interp(rtab + roff[sp], rnr[sp], rdr[sp], r) * r;   // zero at the centre, as phi d_a
+        const double x = r > 0.0 ? dx / r : 0.0, y = r > 0.0 ? dy / r : 0.0, z = r > 0.0 ? dz / r : 0.0;
+        double m;
+        switch (t.M) {
+            case 1: m = current_point<0>(v, phi_total, t.phi0, i, g, x, y, z); break;
+            case 3: m = current_point<1>(v, phi_total, t.phi0, i, g, x, y, z); break;
+            case 5: m = current_point<2>(v, phi_total, t.phi0, i, g, x, y, z); break;
+            default: m = current_point<3>(v, phi_total, t.phi0, i, g, x, y, z); break;
         }
-        const int64_t o = (fn / M) * phi_total + e0 + fn % M;
-        const float hi = __double2float_rn(y);
-        v.phid64[o] = y;
-        v.phid_hi[o] = hi;
-        v.phid_lo[o] = __double2float_rn(y - (double)hi);
+        atomicMax(&top, (unsigned long long)__double_as_longlong(m));
     }
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long*>(peak + t.atom), top);
 }
 
-cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, const double* radial_tab, const int* radial_off,
-                                  const int* radial_nr, const double* radial_dr, cudaStream_t st) {
-    k_current_A<<<(v.natoms + 63) / 64, 64, 0, st>>>(v, T);
-    k_current_tables<<<v.ntiles, TILE, 0, st>>>(v, phi_total, radial_tab, radial_off, radial_nr, radial_dr);
+// The tables scaled, with their FP32 split.
+__global__ void k_current_scale(View v, int64_t phi_total, const double* __restrict__ peak) {
+    const Tile t = v.tiles[blockIdx.x];
+    const double s = current_scale(peak[t.atom]);
+    for (int tab = 0; tab < cur_tables(t.M); ++tab)
+        for (int e = threadIdx.x; e < t.np * t.M; e += blockDim.x) {
+            const int64_t o = tab * phi_total + t.phi0 + e;
+            const double y = v.phid64[o] * s;
+            const float hi = __double2float_rn(y);
+            v.phid64[o] = y;
+            v.phid_hi[o] = hi;
+            v.phid_lo[o] = __double2float_rn(y - (double)hi);
+        }
+}
+
+cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double* T, double* peak, const double* radial_tab,
+                                  const int* radial_off, const int* radial_nr, const double* radial_dr, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(peak, 0, (size_t)v.natoms * sizeof(double), st);
+    if (e != cudaSuccess) return e;
+    k_current_functions<<<v.ntiles, TILE, 0, st>>>(v, phi_total, radial_tab, radial_off, radial_nr, radial_dr, peak);
+    k_current_scale<<<v.ntiles, TILE, 0, st>>>(v, phi_total, peak);
+    static const CurCoupling coupling[4] = {current_coupling<0>(), current_coupling<1>(), current_coupling<2>(), current_coupling<3>()};
+    for (int l = 0; l <= (v.maxM - 1) / 2; ++l)
+        k_current_A<<<(v.natoms * CUR_MAXF + 127) / 128, 128, 0, st>>>(v, l, coupling[l], T, peak);
     return cudaGetLastError();
 }
 
