@@ -318,7 +318,9 @@ dftu_status dftu_import_occupations(dftu_handle h, const double* in, dftu_stream
  * an atomic counter until the list is exhausted, so uneven systems balance themselves.  The small
  * per-system steps (Nbar, occupations, U/J, potential) run as single batched launches.  Results are
  * read per member with the handle calls above (dftu_get_results etc.); the arithmetic is that of the
- * single-system calls, in the same order per member.  The paper has no counterpart for the batching;
+ * single-system calls, in the same order per member at every size (FP32-pair projections of complex128
+ * states: the order of single calls of projection variant 1, since batches run on the 512-point tiles).
+ * The paper has no counterpart for the batching;
  * it packages Eqs. (4)-(11) for many systems at once.  All members must use the same FP64 mode and
  * have no vector potential set (dftu_set_vector_potential); otherwise dftu_batch_project and
  * dftu_batch_apply return DFTU_ERR_INVALID_ARG. */

@@ -31,6 +31,12 @@ bool smem_configured(const void* fn, int bytes) {
 // tiles per atom, 512 states, 64 orbitals: 45.8 -> 26.0 us; 64 atoms, 256 states: 37 -> 34 us.)
 constexpr int RED_BANDS = 32, RED_SLICES = CTA / RED_BANDS, RED_LD = RED_BANDS + 1;
 
+// acc += ph s, rounded alike in both forms of the reduce.
+__device__ __forceinline__ void add_segment(double2& acc, double2 ph, double2 s) {
+    acc.x = fma(ph.x, s.x, fma(-ph.y, s.y, acc.x));
+    acc.y = fma(ph.x, s.y, fma(ph.y, s.x, acc.y));
+}
+
 template <int M>
 __device__ __forceinline__ void reduce_atom(const View& v, int nbands, int ks, int a, int band0, int table, int64_t p_stride, double2* sm) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -48,8 +54,7 @@ __device__ __forceinline__ void reduce_atom(const View& v, int nbands, int ks, i
     auto flush = [&]() {
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            acc[m].x += ph.x * s[m].x - ph.y * s[m].y;
-            acc[m].y += ph.x * s[m].y + ph.y * s[m].x;
+            add_segment(acc[m], ph, s[m]);
             s[m] = make_double2(0.0, 0.0);
         }
     };
@@ -122,38 +127,58 @@ __global__ void __launch_bounds__(CTA, 2) k_tile_reduce(View v, int nbands) {
     reduce_item(v, nbands, blockIdx.x, 0, 0);
 }
 
-// The same sums with a thread per (k*spin, orbital, band), band fastest, walking the atom's tiles in order.  Where the
-// form above takes more than two waves, the SMs are full either way and this one holds more warps: 512 CTAs of the form
-// above 37 (this) against 33 us, 1024 CTAs 31 against 40, 2048 CTAs 64 against 84.
+// The same sums in the same order with a thread per (k*spin, orbital, band), band fastest, walking the atom's tiles
+// range by range: a state's bits do not depend on the size of the call, nor on whether it runs in a batch (which takes
+// the form above).  Where that form takes more than two waves, the SMs are full either way and this one holds more
+// warps: 512 CTAs of the form above 37 (this) against 33 us, 1024 CTAs 31 against 40, 2048 CTAs 64 against 84 (measured
+// with one sum per atom; the ranges changed whole projections of 1024 and 2048 oxide states by -4 and +3 us).
 __global__ void k_tile_reduce_states(View v, int nbands) {
     dependent_release();
     dependent_wait();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= (int64_t)v.nk * v.ns * v.MT * nbands) return;
     const int band = (int)(g % nbands), j = (int)(g / nbands % v.MT), ks = (int)(g / nbands / v.MT);
-    const int a = v.orb_atom[j], m = j - v.atom_moff[a];
-    const double2* part = v.part + ((int64_t)ks * v.TM + m) * v.max_bands + band;
+    const int a = v.orb_atom[j], m = j - v.atom_moff[a], M = v.atom_M[a];
+    const int t0 = v.atom_tile_beg[a], t1 = v.atom_tile_end[a], per = (t1 - t0 + RED_SLICES - 1) / RED_SLICES;
+    const double2* part = v.part + ((int64_t)ks * v.TM + v.tiles[t0].moff + m) * v.max_bands + band;
     const double2* phase = v.seg_phase + ks / v.ns;
-    double2 sum = make_double2(0.0, 0.0), in_seg = sum;
-    int seg = -1;
-    auto close_segment = [&]() {
-        if (seg < 0) return;
-        const double2 ph = phase[(int64_t)seg * v.nk];
-        sum.x += ph.x * in_seg.x - ph.y * in_seg.y;
-        sum.y += ph.x * in_seg.y + ph.y * in_seg.x;
-    };
-    for (int t = v.atom_tile_beg[a]; t < v.atom_tile_end[a]; ++t) {
-        const Tile& tl = v.tiles[t];
-        if (tl.seg != seg) {
-            close_segment();
-            seg = tl.seg;
-            in_seg = make_double2(0.0, 0.0);
+    double2 sum = make_double2(0.0, 0.0), range = sum, in_seg = sum;
+    int seg = v.tiles[t0].seg, end = t0 + per;   // open segment; end of the open range
+    double2 ph = phase[(int64_t)seg * v.nk];
+    constexpr int B = 6;                         // tiles in flight
+    for (int t = t0; t < t1; t += B) {
+        double2 x[B];
+        int sg[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const bool on = t + u < t1;
+            sg[u] = on ? v.tiles[t + u].seg : -1;
+            x[u] = on ? part[(int64_t)(t + u - t0) * M * v.max_bands] : make_double2(0.0, 0.0);
         }
-        const double2 x = part[(int64_t)tl.moff * v.max_bands];
-        in_seg.x += x.x;
-        in_seg.y += x.y;
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            if (t + u >= t1) break;
+            if (sg[u] != seg || t + u == end) {
+                add_segment(range, ph, in_seg);
+                in_seg = make_double2(0.0, 0.0);
+                if (sg[u] != seg) {
+                    seg = sg[u];
+                    ph = phase[(int64_t)seg * v.nk];
+                }
+                if (t + u == end) {
+                    sum.x += range.x;
+                    sum.y += range.y;
+                    range = make_double2(0.0, 0.0);
+                    end += per;
+                }
+            }
+            in_seg.x += x[u].x;
+            in_seg.y += x[u].y;
+        }
     }
-    close_segment();
+    add_segment(range, ph, in_seg);
+    sum.x += range.x;
+    sum.y += range.y;
     sum.x *= v.dV;
     sum.y *= v.dV;
     if (!isfinite(sum.x) || !isfinite(sum.y)) atomicOr(v.status, ST_NONFINITE);
