@@ -236,7 +236,7 @@ cudaError_t launch_project(const View& v, const void* psi, dftu_prec prec, dftu_
     if (gauge) {   // one shape per arithmetic policy with the gauge phases (Sec. V)
         if (prec == DFTU_C64) e = run_project<P_F32, 8, 16, 8, 0, 2, 1>(v, a, st);
         else if (mode == DFTU_F64_NATIVE) e = run_project<P_F64, 8, 1, 4, 0, 2, 1>(v, a, st);
-        else e = run_project<P_PAIR, 8, 8, 8, 5, 2, 1>(v, a, st);
+        else e = run_project<P_PAIR, 8, 8, 8, 5, 2, 1, 1, CTA, TILE, false, true>(v, a, st);
     } else if (prec == DFTU_C64) {
         e = project_f32(v, a, variant, st, &vp);
     } else if (mode == DFTU_F64_NATIVE) {
@@ -270,7 +270,7 @@ cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, 
     // the fixed shapes of the gauge path, with and without the phases
     if (prec == DFTU_C64) e = gauge ? run_project<P_F32, 8, 16, 8, 0, 2, 1, 3>(v, a, st) : run_project<P_F32, 8, 16, 8, 0, 2, 0, 3>(v, a, st);
     else if (mode == DFTU_F64_NATIVE) e = gauge ? run_project<P_F64, 8, 1, 4, 0, 2, 1, 3>(v, a, st) : run_project<P_F64, 8, 1, 4, 0, 2, 0, 3>(v, a, st);
-    else e = gauge ? run_project<P_PAIR, 8, 8, 8, 5, 2, 1, 3>(v, a, st) : run_project<P_PAIR, 8, 8, 8, 5, 2, 0, 3>(v, a, st);
+    else e = gauge ? run_project<P_PAIR, 8, 8, 8, 5, 2, 1, 3, CTA, TILE, false, true>(v, a, st) : run_project<P_PAIR, 8, 8, 8, 5, 2, 0, 3, CTA, TILE, false, true>(v, a, st);
     if (e != cudaSuccess) return e;
     View vd = v;
     vd.p = p_out;

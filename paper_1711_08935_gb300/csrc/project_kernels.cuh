@@ -577,15 +577,17 @@ __host__ __device__ constexpr size_t phi_row_bytes(int pol, int maxM) {
 }
 
 // The bands of one group, [band0, band0 + NT/Q * bands per lane), over the staged tile.  more: a full group of the
-// same shape follows.
-template <int POL, int Q, int CH, int PF, int G, int NT, int TP>
-__device__ __forceinline__ void project_group(const View& v, const Tile& t, const ProjArgs& a, int ks, int band0, bool more, int pe,
+// same shape follows.  HOIST: what comes from outside the loop over groups (1: k and s, 2: the orbitals' exponent); the
+// kernels sit at the register limit of their occupancy, and each form keeps its registers one way only (2048 oxide
+// states: eight groups fixed 2079 us with 1 against 2113, complex64 with 0 1093 against 1112).
+template <int POL, int Q, int CH, int PF, int G, int NT, int TP, int HOIST>
+__device__ __forceinline__ void project_group(const View& v, const Tile& t, const ProjArgs& a, int ks, int k0, int s0, int band0, bool more, const int* s_pe, int pe0,
                                               const unsigned char* smem, const unsigned char* s_gauge, int64_t poff) {
     const int* s_idx = reinterpret_cast<const int*>(smem);
     constexpr int NBL = LaneBands<POL>::value;   // bands per lane
     constexpr int BPW = (32 / Q) * NBL;
     constexpr int BPC = (NT / 32) * BPW;
-    const int k = ks / v.ns, s = ks % v.ns;
+    const int k = HOIST == 1 ? k0 : ks / v.ns, s = HOIST == 1 ? s0 : ks % v.ns;
     const int band = band0 + (threadIdx.x >> 5) * BPW + ((threadIdx.x & 31) / Q) * NBL;
     const bool active = band < a.nbands;
     const int64_t off = (int64_t)k * a.sk + (int64_t)s * a.ss + (int64_t)band * a.sn;
@@ -615,6 +617,7 @@ __device__ __forceinline__ void project_group(const View& v, const Tile& t, cons
         const float4* s_phi = reinterpret_cast<const float4*>(smem + TP * sizeof(int));
         const double2* row = active ? reinterpret_cast<const double2*>(a.psi) + off : nullptr;
         const double2* row_next = (active && more && band + BPC < a.nbands) ? row + (int64_t)BPC * a.sn : nullptr;
+        const int pe = HOIST == 2 ? pe0 : *s_pe;
         const float4* s_g = reinterpret_cast<const float4*>(s_gauge);
         switch (t.M) {
             case 1: proj_body_pair<1, Q, CH, PF, G>(v, t, ks, band, row, row_next, s_idx, s_phi, pe, s_g, poff); break;
@@ -640,12 +643,13 @@ __device__ __forceinline__ void project_group(const View& v, const Tile& t, cons
 // onto several tables).  The tile is staged in shared memory once.  TP: the tiling's largest tile (TILE,
 // or PTILE when the launch's View carries the projection's own tiling); shared memory holds TP grid
 // indices, then TP + 128 orbital rows (zeros past the tile), then the gauge phases.
-template <int POL, int Q, int CH, int NBG, int PF, int G, int NT = CTA, int TP = TILE>
+template <int POL, int Q, int CH, int NBG, int PF, int G, int NT = CTA, int TP = TILE, int TAIL = 0>
 __device__ __forceinline__ void project_item(const View& v, const ProjArgs& a, int tile_id, int ks, int chunk, int nbg,
                                              unsigned char* smem, int* s_pe, int dir = 0) {
     int* s_idx = reinterpret_cast<int*>(smem);
     if (G) dependent_wait();   // the phase table may be the kernel before's
     const Tile t = v.tiles[tile_id];
+    const int k = ks / v.ns, s = ks % v.ns;
     const int64_t ph0 = t.phi0 + dir * v.phi_dir_stride;   // this table's rows of the tile
     const int64_t poff = dir * v.part_dir_stride;
     constexpr int NBL = LaneBands<POL>::value;   // bands per lane
@@ -697,34 +701,32 @@ __device__ __forceinline__ void project_item(const View& v, const ProjArgs& a, i
     __syncthreads();
 
     // ---- stream nbg groups of BPC bands over the staged tile
-    // A last group with few bands takes more lanes per band: its chains get shorter instead of warps idling
+    // TAIL: a last group with few bands takes more lanes per band: its chains get shorter instead of warps idling
     // (65 complex128 bands are two groups of 32 and one of one band, which used to cost as much as a full one).
-    // Only in the default shapes; the split depends on the band count alone, so every launch of a shape sums in
-    // the same order.
     dependent_wait();   // the states
-    constexpr bool TAIL = POL == P_PAIR && Q == 8 && CH == 8 && (PF == 5 || PF == 1);   // (the complex64 kernel would spill)
-    const int pe = *s_pe;
+    constexpr int HOIST = POL != P_PAIR ? 0 : !TAIL ? (NBG != 0) : NBG == 0 ? 2 : 0;
+    const int pe = HOIST == 2 ? *s_pe : 0;
     const int ng = NBG ? NBG : nbg;
     for (int g = 0; g < ng; ++g) {
         const int band0 = (chunk * ng + g) * BPC;
         if (band0 >= a.nbands) break;
         const int left = a.nbands - band0;
-        if (TAIL && Q == 8 && left <= BPC / 4) project_group<POL, TAIL ? 32 : Q, TAIL ? 4 : CH, 0, G, NT, TP>(v, t, a, ks, band0, false, pe, smem, s_gauge, poff);
-        else if (TAIL && left <= BPC / 2) project_group<POL, TAIL ? 2 * Q : Q, TAIL ? 128 / (2 * Q) : CH, 0, G, NT, TP>(v, t, a, ks, band0, false, pe, smem, s_gauge, poff);
-        else project_group<POL, Q, CH, PF, G, NT, TP>(v, t, a, ks, band0, g + 1 < ng, pe, smem, s_gauge, poff);
+        if (TAIL && left <= BPC / 4) project_group<POL, TAIL ? 32 : Q, TAIL ? 4 : CH, 0, G, NT, TP, HOIST>(v, t, a, ks, k, s, band0, false, s_pe, pe, smem, s_gauge, poff);
+        else if (TAIL && left <= BPC / 2) project_group<POL, TAIL ? 16 : Q, TAIL ? 8 : CH, 0, G, NT, TP, HOIST>(v, t, a, ks, k, s, band0, false, s_pe, pe, smem, s_gauge, poff);
+        else project_group<POL, Q, CH, PF, G, NT, TP, HOIST>(v, t, a, ks, k, s, band0, g + 1 < ng, s_pe, pe, smem, s_gauge, poff);
     }
 }
 
 // NDIR > 1: blockIdx.x = tile * NDIR + table, so the CTAs of one tile and band chunk for the
 // NDIR orbital tables are neighbours in the launch and read the same states while they sit in L2.
-template <int POL, int Q, int CH, int NBG, int PF, int MINB, int G, int NDIR = 1, int NT = CTA, int TP = TILE>
+template <int POL, int Q, int CH, int NBG, int PF, int MINB, int G, int NDIR = 1, int NT = CTA, int TP = TILE, int TAIL = 0>
 __global__ void __launch_bounds__(NT, MINB) k_project(View v, ProjArgs a, int nbg) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_pe;
     const int tile = (NDIR == 1) ? (int)blockIdx.x : (int)blockIdx.x / NDIR;
     const int dir = (NDIR == 1) ? 0 : (int)blockIdx.x % NDIR;
     if (NDIR > 1 && dir >= cur_tables(v.tiles[tile].M)) return;   // the atom has fewer tables
-    project_item<POL, Q, CH, NBG, PF, G, NT, TP>(v, a, tile, blockIdx.z, blockIdx.y, nbg, smem, &s_pe, dir);
+    project_item<POL, Q, CH, NBG, PF, G, NT, TP, TAIL>(v, a, tile, blockIdx.z, blockIdx.y, nbg, smem, &s_pe, dir);
 }
 
 // Persistent form over many systems: every CTA takes (system, tile, k*spin) items from a counter until
@@ -763,10 +765,8 @@ inline int balanced_groups(int most, int bands_per_group, int nbands, int64_t ti
     double least = 1e300;
     for (int g = std::min(most, groups); g >= 1; --g) {
         const int64_t ctas = tiles * ((groups + g - 1) / g);
-        const int64_t waves = (ctas + slots - 1) / slots;
-        // beyond a few waves the last one's idle SMs are shared out by the earlier ones
-        const double w = ctas >= 4 * slots ? (double)ctas / slots : (double)waves;
-        const double cost = w * (0.35 + g);
+        // beyond a few waves the SMs share the work out whatever the split: every CTA's staging and every group once
+        const double cost = ctas >= 4 * slots ? (ctas * 0.35 + (double)tiles * groups) / slots : (double)((ctas + slots - 1) / slots) * (0.35 + g);
         if (cost < 0.97 * least) { least = cost; best = g; }
     }
     return best;
@@ -777,25 +777,43 @@ inline int balanced_groups(int most, int bands_per_group, int nbands, int64_t ti
 // the launch ran with, whose tiling the tile reduce must follow.
 // BAL: the band groups per CTA follow the grid, up to NBG (at run time for the FP32-pair kernel; the complex64 kernel
 // spills with a run-time count and is compiled for NBG, NBG / 2 and 1).
-template <int POL, int Q, int CH, int NBG, int PF, int MINB = 2, int G = 0, int NDIR = 1, int NT = CTA, int TP = TILE, bool BAL = false>
+// RAGGED: a last group at most half full may take the kernel in which such groups have more lanes per band.  The
+// three forms are kernels of their own, because the others' code costs the full groups registers that spill: 2048 oxide
+// states take 2079 us with eight groups fixed, 2111 with the count at run time and ragged groups in the kernel.  So
+// - eight groups fixed where that is the split (232 bands, four k: 1932 us against 1951 with the ragged form);
+// - with a balanced split below that, the ragged form (40, 72 and 136 bands: 423, 681 and 1185 us against 461, 704 and
+//   1205; half full groups are equal);
+// - under a vector potential and for the current, eight groups fixed at any size, the ragged form where the last group
+//   counts for much (40, 65 and 264 bands: 527, 788 and 2859 against 562, 821 and 2939; 80 and 112 bands would take
+//   944 and 1284 against 933 and 1262).
+template <int POL, int Q, int CH, int NBG, int PF, int MINB = 2, int G = 0, int NDIR = 1, int NT = CTA, int TP = TILE, bool BAL = false,
+          bool RAGGED = false>
 static cudaError_t run_project(const View& v, const ProjArgs& a, cudaStream_t st, View* used = nullptr) {
     static_assert(Q * CH <= TILE_PAD - TILE, "chained loops read up to Q*CH rows past the tile");
     static_assert(TP == TILE || TP == PTILE, "a tiling the View carries");
+    static_assert(!RAGGED || (POL == P_PAIR && Q == 8 && CH == 8), "the ragged groups' shapes");
     constexpr int TPAD = TP + (TILE_PAD - TILE);
     size_t smem = TP * sizeof(int) + (size_t)TPAD * phi_row_bytes(POL, v.maxM) + (G ? (size_t)TPAD * 16 : 0);
-    auto fn = k_project<POL, Q, CH, (BAL && POL == P_PAIR) ? 0 : NBG, PF, MINB, G, NDIR, NT, TP>;
+    auto fn = k_project<POL, Q, CH, NBG, PF, MINB, G, NDIR, NT, TP>;
     View vl = v;
     if (TP != TILE) {
-        if (!fits_per_sm((const void*)fn, NT, smem, MINB)) return run_project<POL, Q, CH, NBG, PF, MINB, G, NDIR, NT, TILE, BAL>(v, a, st, used);
+        if (!fits_per_sm((const void*)fn, NT, smem, MINB)) return run_project<POL, Q, CH, NBG, PF, MINB, G, NDIR, NT, TILE, BAL, RAGGED>(v, a, st, used);
         vl.tiles = v.ptiles; vl.ntiles = v.nptiles; vl.TM = v.pTM;
         vl.atom_tile_beg = v.patom_tile_beg; vl.atom_tile_end = v.patom_tile_end;
     }
     if (used) *used = vl;
+    constexpr int BPC = (NT / 32) * (32 / Q) * LaneBands<POL>::value;
+    const int nbg = BAL ? balanced_groups(NBG, BPC, a.nbands, (int64_t)vl.ntiles * NDIR * vl.nk * vl.ns, MINB * sm_count()) : NBG;
+    if constexpr (BAL && POL == P_PAIR)
+        if (nbg != NBG) fn = k_project<POL, Q, CH, 0, PF, MINB, G, NDIR, NT, TP>;
+    if constexpr (RAGGED) {
+        const int left = a.nbands % BPC, groups = (a.nbands + BPC - 1) / BPC;
+        const bool pays = BAL ? nbg != NBG : NBG == 1 || groups == 1 || (left <= BPC / 4 && (groups <= 3 || groups % NBG == 1));
+        if (left > 0 && left <= BPC / 2 && pays) fn = k_project<POL, Q, CH, BAL ? 0 : NBG, PF, MINB, G, NDIR, NT, TP, 1>;
+    }
     cudaError_t e = cudaSuccess;
     if (!smem_configured((const void*)fn, (int)smem)) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    constexpr int BPC = (NT / 32) * (32 / Q) * LaneBands<POL>::value;
-    const int nbg = BAL ? balanced_groups(NBG, BPC, a.nbands, (int64_t)vl.ntiles * NDIR * vl.nk * vl.ns, MINB * sm_count()) : NBG;
     dim3 grid(vl.ntiles * NDIR, (a.nbands + BPC * nbg - 1) / (BPC * nbg), vl.nk * vl.ns);
     return launch_dependent(fn, grid, NT, smem, st, vl, a, nbg);
 }
@@ -805,7 +823,7 @@ static cudaError_t run_project(const View& v, const ProjArgs& a, cudaStream_t st
 template <int POL, int Q, int CH, int NBG, int PF, int MINB, int NT, int TP>
 static cudaError_t run_project_default(const View& v, const ProjArgs& a, cudaStream_t st, View* used) {
     if constexpr (POL == P_PAIR) {
-        return run_project<POL, Q, CH, NBG, PF, MINB, 0, 1, NT, TP, true>(v, a, st, used);
+        return run_project<POL, Q, CH, NBG, PF, MINB, 0, 1, NT, TP, true, true>(v, a, st, used);
     } else {
         constexpr int BPC = (NT / 32) * (32 / Q) * LaneBands<POL>::value;
         const int nbg = balanced_groups(NBG, BPC, a.nbands, (int64_t)v.ntiles * v.nk * v.ns, MINB * sm_count());

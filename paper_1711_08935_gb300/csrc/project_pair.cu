@@ -25,7 +25,7 @@ namespace dftu {
 static cudaError_t project_pair_default(const View& v, const ProjArgs& a, cudaStream_t st, View* used) {
     const int64_t sms = sm_count(), rows = (int64_t)v.nk * v.ns, groups = (a.nbands + 31) / 32;
     if (v.nptiles * groups * rows >= 2 * sms) return run_project_default<DFTU_PROJECT_DEFAULT_PAIR>(v, a, st, used);
-    if (v.ntiles * groups * rows >= sms) return run_project<P_PAIR, 8, 8, 1, 1, 2, 0, 1, 256, TILE>(v, a, st, used);
+    if (v.ntiles * groups * rows >= sms) return run_project<P_PAIR, 8, 8, 1, 1, 2, 0, 1, 256, TILE, false, true>(v, a, st, used);
     return run_project<P_PAIR, 16, 8, 1, 1, 2, 0, 1, 256, TILE>(v, a, st, used);
 }
 
