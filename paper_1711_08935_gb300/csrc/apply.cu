@@ -626,10 +626,15 @@ cudaError_t launch_apply(const View& v, void* psi, dftu_prec prec, dftu_f64_mode
                          int64_t sk, int64_t ss, int64_t sn, const double* coef, const int* color_order,
                          const std::vector<int>& color_beg, int variant, int accumulate, cudaStream_t st, bool gauge) {
     ApplyArgs a{psi, sk, ss, sn, nbands, coef, nullptr, accumulate};
-    if (gauge) {   // one shape per arithmetic policy with the gauge phases (Sec. V)
+    if (gauge) {   // the shapes with the gauge phases (Sec. V)
         if (prec == DFTU_C64) return run_apply<A_F32, 8, 4, 8, 1, 1>(v, a, color_order, color_beg, st);
         if (mode == DFTU_F64_NATIVE) return run_apply<A_F64, 8, 4, 4, 0, 1>(v, a, color_order, color_beg, st);
-        return run_apply<A_PAIR, 16, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
+        // Eight lanes per band (groups of 32 bands), 16 (groups of 16, a ragged last one of 8) where eight would leave most
+        // of the last of at most two groups idle.  16 oxide spheres, four k, us with 8 / 16 lanes: 256 bands 4241 / 4562,
+        // 96 bands 1639 / 1757, 40 bands 805 / 780, 24 bands 487 / 501, 16 bands 375 / 345, 4 bands 252 / 142.
+        const int left = nbands % 32;
+        if (nbands <= 16 || (nbands < 64 && left > 0 && left <= 8)) return run_apply<A_PAIR, 16, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
+        return run_apply<A_PAIR, 8, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
     }
 #define DFTU_CASE_F32(i, POL, Q, NBG, U, PF) case i: return run_apply<POL, Q, NBG, U, PF>(v, a, color_order, color_beg, st);
 #define DFTU_CASE_PAIR(i, Q, NBG, U, PF) case i: return run_apply<A_PAIR, Q, NBG, U, PF>(v, a, color_order, color_beg, st);

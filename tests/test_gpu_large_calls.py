@@ -67,3 +67,26 @@ def test_pair_projections_of_large_calls(nb):
         # relative to the sum of the terms' moduli, here its Cauchy-Schwarz bound over random signs
         assert np.max(np.abs(J[0] - J[1])) <= 1e-11 * np.max(np.abs(J[0]))
     assert h.sync_status() == dftu.DFTU_OK
+
+
+@pytest.mark.parametrize("nb", [16, 17, 32, 33, 40, 41])
+def test_gauge_apply_at_the_band_counts_where_its_shape_changes(nb):
+    """Both lane counts of the FP32-pair gauge scatter against native FP64, with enough rows for the production shape."""
+    s = _system(3 * torch.cuda.get_device_properties(0).multi_processor_count // 2)
+    psi = _random_states(s, nb, seed=nb)
+    f = torch.rand(s.nk, 1, nb, generator=torch.Generator(device="cuda").manual_seed(5), device="cuda", dtype=torch.float64) / nb
+    h = dftu.handle_for_system(s, nb)
+    for I in range(3):
+        h.set_u(I, 0.4, 0.05)
+    h.set_vector_potential(torch.tensor(A, dtype=torch.float64, device="cuda"))
+    out = []
+    h.set_f64_mode(dftu.F64_NATIVE)
+    h.project(psi)
+    h.occupations(f)
+    h.acbn0_uj()
+    for mode in (dftu.F64_NATIVE, dftu.F64_PAIR):
+        h.set_f64_mode(mode)
+        x = psi.clone()
+        h.apply(x)
+        out.append(x)
+    assert float((out[0] - out[1]).abs().max()) < 1e-12 * float(out[0].abs().max())
