@@ -69,6 +69,92 @@ def test_pair_projections_of_large_calls(nb):
     assert h.sync_status() == dftu.DFTU_OK
 
 
+def _apply_bands(s, extra):
+    """Bands for which every colour of an apply, even one with a single tile, passes the small-call threshold (half of
+    three blocks per SM, a block per tile, row and 64 bands), and `extra` more."""
+    chunks = -(-3 * torch.cuda.get_device_properties(0).multi_processor_count // (2 * s.nk * s.nspin))
+    return 64 * chunks + extra
+
+
+def _subset(s, ks):
+    sub = _cases.overlapping_three_atoms()
+    sub.kpts, sub.wk = s.kpts[ks], s.wk[ks]
+    return sub
+
+
+# whole groups, and 5 or 13 bands more (ragged groups of 16 and 32 bands)
+@pytest.mark.parametrize("extra", [0, 5, 13])
+@pytest.mark.parametrize("kind", ["pair", "native", "complex64"])
+@pytest.mark.parametrize("vector_potential", [None, A])
+def test_apply_of_large_calls_matches_oracle(kind, extra, vector_potential):
+    """The production shapes of the scatter, plain and with the gauge phases, in the three arithmetics: bands of the
+    first, a middle and the last group at two k-points against the oracle's apply with the handle's own potential."""
+    s = _system(48)
+    nb = _apply_bands(s, extra)
+    st = O.setup_atoms(s)
+    dtype = torch.complex64 if kind == "complex64" else torch.complex128
+    psi = _random_states(s, nb, seed=extra).to(dtype)
+    f = torch.rand(s.nk, 1, nb, generator=torch.Generator(device="cuda").manual_seed(2), device="cuda", dtype=torch.float64) / nb
+    h = dftu.handle_for_system(s, nb)
+    h.set_f64_mode(dftu.F64_NATIVE if kind == "native" else dftu.F64_PAIR)
+    for I in range(3):
+        h.set_u(I, 0.4, 0.05)
+    if vector_potential is not None:
+        h.set_vector_potential(torch.tensor(vector_potential, dtype=torch.float64, device="cuda"))
+    ks, bands = [0, 47], [0, 1, nb // 2, nb - 14, nb - 6, nb - 2, nb - 1]
+    before = psi[ks][:, :, bands].to(torch.complex128).cpu().numpy()
+    h.project(psi)
+    h.occupations(f)
+    h.acbn0_uj()
+    h.apply(psi)
+    got = psi[ks][:, :, bands].to(torch.complex128).cpu().numpy()
+    V = [0.35 * (0.5 * np.eye(n.shape[-1]) - n.transpose(0, 2, 1)) for n in h.results()["n"]]
+    sub, vec = _subset(s, ks), np.array(vector_potential or (0.0, 0.0, 0.0))
+    ref = O.apply_gauge(sub, st, before, O.project_gauge(sub, st, before, vec), V, vec)
+    assert np.max(np.abs(got - ref)) < (1e-6 if kind == "complex64" else 1e-12) * np.max(np.abs(ref))
+    assert h.sync_status() == dftu.DFTU_OK
+
+
+@pytest.mark.parametrize("extra", [0, 5])
+def test_fused_real_time_steps_of_large_calls_match_oracle(extra):
+    """Three fused complex64 steps whose scatters all take the production shape, on tiles of both kinds (spheres that
+    overlap each other and their own images): states, projections and the handle's potential against the oracle's
+    steps, on sampled bands with the potential of every step formed from all of them by single native FP64 steps."""
+    s = _system(48)
+    nb = _apply_bands(s, extra)
+    st = O.setup_atoms(s)
+    psi = _random_states(s, nb, seed=7 + extra).to(torch.complex64)
+    f = torch.rand(s.nk, 1, nb, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda", dtype=torch.float64) / nb
+    fused, native = dftu.handle_for_system(s, nb), dftu.handle_for_system(s, nb)
+    native.set_f64_mode(dftu.F64_NATIVE)
+    for h in (fused, native):
+        for I in range(3):
+            h.set_u(I, 0.4, 0.05)
+    ks, bands, dt = [0, 47], [0, nb // 2, nb - 6, nb - 2, nb - 1], 0.5
+    sub = _subset(s, ks)
+    ref = psi[ks][:, :, bands].to(torch.complex128).cpu().numpy()
+    t = psi.to(torch.complex128)
+    fused.taylor_steps(psi, f, dt, 3)
+    for _ in range(3):
+        native.taylor_step(t, None, f, dt)
+        V = [0.35 * (0.5 * np.eye(n.shape[-1]) - n.transpose(0, 2, 1)) for n in native.results()["n"]]
+        term = out = ref
+        for j in range(1, 5):
+            term = O.apply(sub, st, np.zeros_like(term), O.project(sub, st, term), V, -1j * dt / j)
+            out = out + term
+        ref = out
+    assert np.max(np.abs(t[ks][:, :, bands].cpu().numpy() - ref)) < 1e-11 * np.max(np.abs(ref))
+    got = psi[ks][:, :, bands].to(torch.complex128).cpu().numpy()
+    assert np.max(np.abs(got - ref)) < 2e-6 * np.max(np.abs(ref))
+    assert float((psi.to(torch.complex128) - t).abs().max()) < 2e-6 * float(t.abs().max())
+    p = fused.projections(nb)[ks][:, bands]
+    p_ref = np.concatenate([x[:, 0] for x in O.project(sub, st, got)], axis=-1)
+    assert np.max(np.abs(p - p_ref)) < 2e-6 * np.max(np.abs(p_ref))
+    for a, b in zip(fused.results()["n"], native.results()["n"]):
+        assert np.max(np.abs(a - b)) < 1e-6 * max(1.0, np.max(np.abs(b)))
+    assert fused.sync_status() == dftu.DFTU_OK
+
+
 @pytest.mark.parametrize("nb", [16, 17, 32, 33, 40, 41])
 def test_gauge_apply_at_the_band_counts_where_its_shape_changes(nb):
     """Both lane counts of the FP32-pair gauge scatter against native FP64, with enough rows for the production shape."""
