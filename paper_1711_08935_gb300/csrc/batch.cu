@@ -24,6 +24,7 @@ struct dftu_batch_ctx {
     int4* d_color_items = nullptr;
     int* d_counter = nullptr;
     std::vector<int> nbands;
+    std::vector<int> order;   // members in the order of the item lists
 };
 
 namespace {
@@ -31,6 +32,45 @@ namespace {
 dftu_status bfail(dftu_batch_ctx* b, dftu_status s, const std::string& m) {
     b->err = m;
     return s;
+}
+
+// Work items of all members, member by member in the given order, and the apply's by colour.
+void list_items(const dftu_batch_ctx* b, const std::vector<int>& order, std::vector<int4>& items, std::vector<int4>& citems,
+                std::vector<int>& color_beg) {
+    int ncol = 0;
+    for (auto* c : b->members) ncol = std::max(ncol, (int)c->color_beg.size() - 1);
+    std::vector<std::vector<int4>> by_color(ncol);
+    items.clear();
+    for (int s : order) {
+        const Ctx* c = b->members[s];
+        const int rows = c->nk * c->ns;
+        for (int t = 0; t < (int)c->tiles.size(); ++t)
+            for (int ks = 0; ks < rows; ++ks) items.push_back(make_int4(s, t, ks, 0));
+        for (int col = 0; col + 1 < (int)c->color_beg.size(); ++col)
+            for (int q = c->color_beg[col]; q < c->color_beg[col + 1]; ++q)
+                for (int ks = 0; ks < rows; ++ks) by_color[col].push_back(make_int4(s, c->color_order[q], ks, 0));
+    }
+    citems.clear();
+    color_beg.assign(1, 0);
+    for (auto& v : by_color) {
+        citems.insert(citems.end(), v.begin(), v.end());
+        color_beg.push_back((int)citems.size());
+    }
+}
+
+cudaError_t upload_items(dftu_batch_ctx* b, const std::vector<int4>& items, const std::vector<int4>& citems) {
+    cudaFree(b->d_items);
+    cudaFree(b->d_color_items);
+    b->d_items = b->d_color_items = nullptr;
+    cudaError_t e = cudaMalloc(&b->d_items, items.size() * sizeof(int4));
+    if (e == cudaSuccess) e = cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_color_items, std::max<size_t>(1, citems.size()) * sizeof(int4));
+    if (e == cudaSuccess && !citems.empty())
+        e = cudaMemcpy(b->d_color_items, citems.data(), citems.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    b->L.items = b->d_items;
+    b->L.nitems = (int)items.size();
+    b->L.color_items = b->d_color_items;
+    return e;
 }
 
 void free_tables(dftu_batch_ctx* b) {
@@ -63,48 +103,27 @@ dftu_status dftu_batch_create(dftu_batch* out, int nsys, const dftu_handle* syst
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
     std::vector<View> views;
-    std::vector<int4> items;
-    int ncol = 0;
-    for (auto* c : b->members) ncol = std::max(ncol, (int)c->color_beg.size() - 1);
-    std::vector<std::vector<int4>> by_color(ncol);
     BatchLaunch& L = b->L;
     L.nsys = nsys;
     L.maxM = 1;
     L.max_atoms = 1;
     L.max_ns = 1;
-    for (auto* c : b->members) views.push_back(c->v);
-    // The persistent kernels take items in this order; a system's items all take its whole band count, so the systems
-    // with the most bands come first and the short items fill the end of the launch.
-    std::vector<int> order(nsys);
-    for (int s = 0; s < nsys; ++s) order[s] = s;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->members[x]->max_bands > b->members[y]->max_bands; });
-    for (int s : order) {
+    for (int s = 0; s < nsys; ++s) {
         Ctx* c = b->members[s];
+        views.push_back(c->v);
+        b->order.push_back(s);
         L.maxM = std::max(L.maxM, c->v.maxM);
         L.max_atoms = std::max(L.max_atoms, (int)c->atoms.size());
         L.max_ns = std::max(L.max_ns, c->spin == DFTU_NONCOLLINEAR ? 1 : c->ns);
-        const int rows = c->nk * c->ns;
-        for (int t = 0; t < (int)c->tiles.size(); ++t)
-            for (int ks = 0; ks < rows; ++ks) items.push_back(make_int4(s, t, ks, 0));
-        for (int col = 0; col + 1 < (int)c->color_beg.size(); ++col)
-            for (int q = c->color_beg[col]; q < c->color_beg[col + 1]; ++q)
-                for (int ks = 0; ks < rows; ++ks) by_color[col].push_back(make_int4(s, c->color_order[q], ks, 0));
     }
-    std::vector<int4> citems;
-    L.color_beg.assign(1, 0);
-    for (auto& v : by_color) {
-        citems.insert(citems.end(), v.begin(), v.end());
-        L.color_beg.push_back((int)citems.size());
-    }
+    std::vector<int4> items, citems;
+    list_items(b, b->order, items, citems, L.color_beg);
+    const size_t ncol = L.color_beg.size() - 1;
     cudaError_t e = cudaMalloc(&b->d_views, views.size() * sizeof(View));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_views, views.data(), views.size() * sizeof(View), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_items, items.size() * sizeof(int4));
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_color_items, std::max<size_t>(1, citems.size()) * sizeof(int4));
-    if (e == cudaSuccess && !citems.empty())
-        e = cudaMemcpy(b->d_color_items, citems.data(), citems.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload_items(b, items, citems);
     // one queue counter per launch of an apply (its colours), so that one memset serves them all
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, std::max<size_t>(1, (size_t)ncol) * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, std::max<size_t>(1, ncol) * sizeof(int));
     if (prev >= 0) cudaSetDevice(prev);
     if (e != cudaSuccess) {
         cudaFree(b->d_views); cudaFree(b->d_items); cudaFree(b->d_color_items); cudaFree(b->d_counter);
@@ -112,9 +131,6 @@ dftu_status dftu_batch_create(dftu_batch* out, int nsys, const dftu_handle* syst
         return e == cudaErrorMemoryAllocation ? DFTU_ERR_ALLOC : DFTU_ERR_CUDA;
     }
     L.views = b->d_views;
-    L.items = b->d_items;
-    L.nitems = (int)items.size();
-    L.color_items = b->d_color_items;
     L.counter = b->d_counter;
     *out = b;
     return DFTU_OK;
@@ -149,11 +165,27 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
         max_ctas = std::max<int64_t>(max_ctas, (int64_t)c->nk * c->ns * ((nbands[s] + 31) / 32) * (int64_t)c->atoms.size());
         max_rows = std::max(max_rows, (c->spin == DFTU_NONCOLLINEAR ? c->nk : c->nk * c->ns) * nbands[s] * c->nspecies);
     }
+    // The persistent kernels take items in list order; a member's items all take its bound bands, so the members with the
+    // most bands come first and the short items fill the end of a launch.  Only a bind that changes the order rewrites
+    // the lists.
+    std::vector<int> order(n);
+    for (int s = 0; s < n; ++s) order[s] = s;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return nbands[x] > nbands[y]; });
+    std::vector<int4> items, citems;
+    std::vector<int> color_beg;   // as at creation: the colours do not depend on the order
+    if (order != b->order) list_items(b, order, items, citems, color_beg);
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
+    b->bound = false;   // until the new tables stand
     free_tables(b);
-    cudaError_t e = cudaMalloc(&b->d_args, n * sizeof(ProjArgs));
+    cudaError_t e = cudaSuccess;
+    if (order != b->order) {   // replaced like the tables above: freeing them waits for the launches that read them
+        b->order.clear();
+        e = upload_items(b, items, citems);
+        if (e == cudaSuccess) b->order = order;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_args, n * sizeof(ProjArgs));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_args, args.data(), n * sizeof(ProjArgs), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_f, n * sizeof(double*));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_f, f, n * sizeof(double*), cudaMemcpyHostToDevice);

@@ -54,3 +54,36 @@ def test_wide_members_of_a_batch_are_single_calls_bitwise(dtype, mode):
         assert all(np.array_equal(p, q) for p, q in zip(ra["n"], rb["n"])) and ra["EU"] == rb["EU"]
         assert torch.equal(x, y)
     batch.close()
+
+
+def test_rebinding_with_other_band_counts():
+    """Members of one capacity bound to ascending, then to descending band counts (the item lists follow the bound
+    counts, longest first), complex64: every bind gives each member the bits of the same calls made alone."""
+    s = _cases.overlapping_three_atoms()
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    members = [dftu.handle_for_system(s, 90) for _ in range(3)]
+    alone = dftu.handle_for_system(s, 90)
+    for h in members + [alone]:
+        for I in range(3):
+            h.set_u(I, 0.4, 0.05)
+    batch = dftu.Batch(members)
+    for counts in ((3, 40, 90), (90, 40, 3), (40, 90, 3)):
+        psis = [torch.view_as_complex(torch.randn(s.nk, 1, nb, s.grid.npts, 2, generator=gen, device="cuda")) for nb in counts]
+        fs = [torch.rand(s.nk, 1, nb, generator=gen, device="cuda", dtype=torch.float64) / nb for nb in counts]
+        refs = []
+        for x, f in zip(psis, fs):
+            y = x.clone()
+            alone.project(y)
+            alone.occupations(f)
+            alone.acbn0_uj()
+            alone.apply(y)
+            refs.append((y, alone.results()["EU"]))
+        batch.bind(psis, fs)
+        batch.project()
+        batch.occupations()
+        batch.acbn0_uj()
+        batch.apply()
+        torch.cuda.synchronize()
+        for h, x, (y, e) in zip(members, psis, refs):
+            assert torch.equal(x, y) and h.results()["EU"] == e
+    batch.close()
