@@ -630,12 +630,14 @@ cudaError_t launch_apply(const View& v, void* psi, dftu_prec prec, dftu_f64_mode
     if (gauge) {   // the shapes with the gauge phases (Sec. V)
         if (prec == DFTU_C64) return run_apply<A_F32, 8, 4, 8, 1, 1>(v, a, color_order, color_beg, st);
         if (mode == DFTU_F64_NATIVE) return run_apply<A_F64, 8, 4, 4, 0, 1>(v, a, color_order, color_beg, st);
-        // Eight lanes per band (groups of 32 bands), 16 (groups of 16, a ragged last one of 8) where eight would leave most
-        // of the last of at most two groups idle.  16 oxide spheres, four k, us with 8 / 16 lanes: 256 bands 4241 / 4562,
-        // 96 bands 1639 / 1757, 40 bands 805 / 780, 24 bands 487 / 501, 16 bands 375 / 345, 4 bands 252 / 142.
+        // 64 bands per CTA: two groups of 32 with eight lanes per band, four groups of 16 with 16 (a ragged last one of 8)
+        // where eight would leave most of the last of at most two groups idle.  Us with 8 / 16 lanes, 16 oxide spheres and
+        // four k: 256 bands 4188 / 4557, 96 bands 1626 / 1758, 24 bands 487 / 502, 40 bands 804 / 781, 16 bands 375 / 345,
+        // 4 bands 252 / 142; 64 overlapping spheres, 96 bands: 324 / 351 (372 with 128 bands per CTA: the later colours'
+        // grids are small).
         const int left = nbands % 32;
         if (nbands <= 16 || (nbands < 64 && left > 0 && left <= 8)) return run_apply<A_PAIR, 16, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
-        return run_apply<A_PAIR, 8, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
+        return run_apply<A_PAIR, 8, 2, 4, 1, 1>(v, a, color_order, color_beg, st);
     }
 #define DFTU_CASE_F32(i, POL, Q, NBG, U, PF) case i: return run_apply<POL, Q, NBG, U, PF>(v, a, color_order, color_beg, st, true);
 #define DFTU_CASE_PAIR(i, Q, NBG, U, PF) case i: return run_apply<A_PAIR, Q, NBG, U, PF>(v, a, color_order, color_beg, st, true);
