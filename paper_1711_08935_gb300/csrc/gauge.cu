@@ -87,7 +87,8 @@ cudaError_t launch_gauge_phases(const View& v, const double* A, cudaStream_t st)
 // unpolarised states.
 // An atom's states are split over CUR_SPLIT CTAs, and a CTA takes CUR_STATES states at a time, a lane each; its four
 // warps share the rows of t (through shared memory) and the functions f.  Few states, few warps: the FP64 pipe of one
-// SM quarter, 80 cycles an instruction of a warp, would bound a thread per state.
+// SM quarter, 80 cycles an instruction of a warp, would bound a thread per state.  16 atoms, 192 states: 12.8 us from
+// cold caches (12.3 for the monomials with a thread per state, 60 % of the operations; 19.3 for the displaced orbitals).
 constexpr int CUR_STATES = 32, CUR_PARTS = 4;
 
 template <int M>

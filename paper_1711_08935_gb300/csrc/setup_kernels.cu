@@ -175,6 +175,7 @@ __host__ __device__ __forceinline__ void neighbour_harmonics(double x, double y,
 
 // n_a Y_lm = sum_f c[a][m][f] Y_f over the harmonics f of degree l + 1 (first) and l - 1.
 struct CurCoupling { double c[3][MAXM][CUR_MAXF]; };
+struct CurCouplings { CurCoupling of[4]; };   // by l (9.4 KB of kernel arguments)
 
 // The integrals of n_a Y_lm Y_f over the sphere, by six Gauss-Legendre points in z and twelve angles (exact to degree
 // 11; the products have degree 2l + 2 <= 8).
@@ -211,11 +212,13 @@ static CurCoupling current_coupling() {
 
 __device__ __forceinline__ double current_scale(double peak) { return peak > 0.0 ? (1.0 - 0x1p-20) / peak : 1.0; }
 
-// A[f][a][m] of every atom of degree l: phi_m d_a = sum_f A[f][a][m] F_f.  One thread per (atom, f).
-__global__ void k_current_A(View v, int l, CurCoupling C, const double* __restrict__ T, const double* __restrict__ peak) {
+// A[f][a][m] of every atom: phi_m d_a = sum_f A[f][a][m] F_f.  One thread per (atom, f).
+__global__ void k_current_A(View v, const __grid_constant__ CurCouplings all, const double* __restrict__ T, const double* __restrict__ peak) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    const int a = g / CUR_MAXF, f = g % CUR_MAXF, M = 2 * l + 1;
-    if (a >= v.natoms || v.atom_M[a] != M || f >= cur_functions(M)) return;
+    const int a = g / CUR_MAXF, f = g % CUR_MAXF;
+    if (a >= v.natoms || f >= cur_functions(v.atom_M[a])) return;
+    const int M = v.atom_M[a];
+    const CurCoupling& C = all.of[(M - 1) / 2];
     const double un = 1.0 / current_scale(peak[a]);
     for (int d = 0; d < 3; ++d)
         for (int m = 0; m < M; ++m) {
@@ -225,23 +228,25 @@ __global__ void k_current_A(View v, int l, CurCoupling C, const double* __restri
         }
 }
 
-// The functions of one point, g times the harmonics; returns the largest magnitude.
+// The functions of one point, g times the harmonics; returns the bits of the largest magnitude, which order like the
+// numbers (a comparison off the FP64 pipe, which bounds this kernel).
 template <int l>
-__device__ __forceinline__ double current_point(const View& v, int64_t phi_total, int64_t phi0, int i, double g, double x, double y, double z) {
+__device__ __forceinline__ unsigned long long current_point(const View& v, int64_t phi_total, int64_t phi0, int i, double g, double x, double y, double z) {
     constexpr int M = 2 * l + 1;
-    double F[cur_functions(M)], m = 0.0;
+    double F[cur_functions(M)];
+    unsigned long long m = 0;
     neighbour_harmonics<l>(x, y, z, F);
 #pragma unroll
     for (int f = 0; f < cur_functions(M); ++f) {
         const double q = g * F[f];
         v.phid64[(f / M) * phi_total + phi0 + (int64_t)i * M + f % M] = q;
-        m = fmax(m, fabs(q));
+        m = max(m, (unsigned long long)__double_as_longlong(q) & 0x7FFFFFFFFFFFFFFFull);
     }
     return m;
 }
 
-// phid64[table][point][m] = R r times the harmonic numbered table M + m, and the atom's largest magnitude (its bits
-// order like the numbers; peak starts at zero).
+// phid64[table][point][m] = R r times the harmonic numbered table M + m, and the atom's largest magnitude (peak starts at
+// zero).
 __global__ void k_current_functions(View v, int64_t phi_total, const double* __restrict__ rtab, const int* __restrict__ roff,
                                     const int* __restrict__ rnr, const double* __restrict__ rdr, double* __restrict__ peak) {
     __shared__ unsigned long long top;
@@ -258,15 +263,15 @@ __global__ void k_current_functions(View v, int64_t phi_total, const double* __r
         const double dz = __dsub_rn(__dadd_rn(__dmul_rn((double)kz, v.h2), v.o2), v.atom_pos[3 * a + 2]);
         const double r = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
         const double g = radial_interp(rtab + roff[sp], rnr[sp], rdr[sp], r) * r;   // zero at the centre, as phi d_a
-        const double x = r > 0.0 ? dx / r : 0.0, y = r > 0.0 ? dy / r : 0.0, z = r > 0.0 ? dz / r : 0.0;
-        double m;
+        const double inv = r > 0.0 ? 1.0 / r : 0.0, x = dx * inv, y = dy * inv, z = dz * inv;
+        unsigned long long m;
         switch (t.M) {
             case 1: m = current_point<0>(v, phi_total, t.phi0, i, g, x, y, z); break;
             case 3: m = current_point<1>(v, phi_total, t.phi0, i, g, x, y, z); break;
             case 5: m = current_point<2>(v, phi_total, t.phi0, i, g, x, y, z); break;
             default: m = current_point<3>(v, phi_total, t.phi0, i, g, x, y, z); break;
         }
-        atomicMax(&top, (unsigned long long)__double_as_longlong(m));
+        atomicMax(&top, m);
     }
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long*>(peak + t.atom), top);
@@ -274,8 +279,11 @@ __global__ void k_current_functions(View v, int64_t phi_total, const double* __r
 
 // The tables scaled, with their FP32 split.
 __global__ void k_current_scale(View v, int64_t phi_total, const double* __restrict__ peak) {
+    __shared__ double scale;
     const Tile t = v.tiles[blockIdx.x];
-    const double s = current_scale(peak[t.atom]);
+    if (threadIdx.x == 0) scale = current_scale(peak[t.atom]);
+    __syncthreads();
+    const double s = scale;
     for (int tab = 0; tab < cur_tables(t.M); ++tab)
         for (int e = threadIdx.x; e < t.np * t.M; e += blockDim.x) {
             const int64_t o = tab * phi_total + t.phi0 + e;
@@ -293,9 +301,8 @@ cudaError_t launch_current_tables(const View& v, int64_t phi_total, const double
     if (e != cudaSuccess) return e;
     k_current_functions<<<v.ntiles, TILE, 0, st>>>(v, phi_total, radial_tab, radial_off, radial_nr, radial_dr, peak);
     k_current_scale<<<v.ntiles, TILE, 0, st>>>(v, phi_total, peak);
-    static const CurCoupling coupling[4] = {current_coupling<0>(), current_coupling<1>(), current_coupling<2>(), current_coupling<3>()};
-    for (int l = 0; l <= (v.maxM - 1) / 2; ++l)
-        k_current_A<<<(v.natoms * CUR_MAXF + 127) / 128, 128, 0, st>>>(v, l, coupling[l], T, peak);
+    static const CurCouplings couplings{{current_coupling<0>(), current_coupling<1>(), current_coupling<2>(), current_coupling<3>()}};
+    k_current_A<<<(v.natoms * CUR_MAXF + 127) / 128, 128, 0, st>>>(v, couplings, T, peak);
     return cudaGetLastError();
 }
 
