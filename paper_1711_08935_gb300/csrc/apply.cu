@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(CTA, 3) k_apply_batch(const View* __restrict__
 
 template <int POL, int Q, int NBG, int U, int PF, int G = 0>
 static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order, const std::vector<int>& color_beg,
-                             cudaStream_t st, bool as_is = false) {
+                             cudaStream_t st) {
     constexpr int BPC = (CTA / 32) * (32 / Q);
     size_t smem = TILE * sizeof(int) + BPC * MAXM * 16 + (size_t)TILE_PAD * v.maxM * (POL == A_F64 ? sizeof(double) : sizeof(float4)) +
                   (G ? (size_t)TILE_PAD * 16 : 0);
@@ -595,8 +595,7 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
     // A colour with few tiles (where spheres overlap) or a small call leaves SMs idle with NBG groups of bands per
     // CTA, and is then one chain of latencies: below half the GPU's slots it takes one group of 32 lanes per band (one
     // tile, 256 complex64 bands: 34 -> 13 us; 79 tiles, 316 of 456 slots, would slow down: 63 -> 70).  The update of
-    // a point does not depend on the shape (the fused form's FP32 sums of a tile follow the lanes).  as_is: a shape that
-    // was asked for by number runs as it is.
+    // a point does not depend on the shape.
     auto small = k_apply<POL, 32, 1, 4, PF, G>;
     if (!smem_configured((const void*)small, (int)smem)) e = cudaFuncSetAttribute(small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -606,7 +605,7 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
         if (n == 0) continue;
         a.tile_list = color_order + color_beg[c];
         dim3 grid(n, (a.nbands + BPC * NBG - 1) / (BPC * NBG), v.nk * v.ns);
-        if (as_is || 2 * (int64_t)grid.x * grid.y * grid.z >= slots) e = launch_dependent(fn, grid, CTA, smem, st, v, a);
+        if (2 * (int64_t)grid.x * grid.y * grid.z >= slots) e = launch_dependent(fn, grid, CTA, smem, st, v, a);
         else e = launch_dependent(small, dim3(n, (a.nbands + CTA / 32 - 1) / (CTA / 32), v.nk * v.ns), CTA, smem, st, v, a);
         if (e != cudaSuccess) return e;
     }
@@ -639,8 +638,8 @@ cudaError_t launch_apply(const View& v, void* psi, dftu_prec prec, dftu_f64_mode
         if (nbands <= 16 || (nbands < 64 && left > 0 && left <= 8)) return run_apply<A_PAIR, 16, 4, 4, 1, 1>(v, a, color_order, color_beg, st);
         return run_apply<A_PAIR, 8, 2, 4, 1, 1>(v, a, color_order, color_beg, st);
     }
-#define DFTU_CASE_F32(i, POL, Q, NBG, U, PF) case i: return run_apply<POL, Q, NBG, U, PF>(v, a, color_order, color_beg, st, true);
-#define DFTU_CASE_PAIR(i, Q, NBG, U, PF) case i: return run_apply<A_PAIR, Q, NBG, U, PF>(v, a, color_order, color_beg, st, true);
+#define DFTU_CASE_F32(i, POL, Q, NBG, U, PF) case i: return run_apply<POL, Q, NBG, U, PF>(v, a, color_order, color_beg, st);
+#define DFTU_CASE_PAIR(i, Q, NBG, U, PF) case i: return run_apply<A_PAIR, Q, NBG, U, PF>(v, a, color_order, color_beg, st);
     if (prec == DFTU_C64) {
         switch (variant) {
             DFTU_APPLY_SHAPES_F32(DFTU_CASE_F32)
