@@ -594,8 +594,9 @@ static cudaError_t run_apply(const View& v, ApplyArgs a, const int* color_order,
     if (e != cudaSuccess) return e;
     // A colour with few tiles (where spheres overlap) or a small call leaves SMs idle with NBG groups of bands per
     // CTA, and is then one chain of latencies: below half the GPU's slots it takes one group of 32 lanes per band (one
-    // tile, 256 complex64 bands: 34 -> 13 us; 79 tiles, 316 of 456 slots, would slow down: 63 -> 70).  The update of
-    // a point does not depend on the shape.
+    // tile, 256 complex64 bands: 34 -> 13 us; 79 tiles, 316 of 456 slots, would slow down: 63 -> 70), whatever shape was
+    // asked for (128 molecules one by one with the shape that their batch was tuned to: 24.4 ms, 34.3 with that shape as it
+    // is).  The update of a point does not depend on the shape (the fused form's FP32 sums of a tile follow the lanes).
     auto small = k_apply<POL, 32, 1, 4, PF, G>;
     if (!smem_configured((const void*)small, (int)smem)) e = cudaFuncSetAttribute(small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -176,3 +176,29 @@ def test_gauge_apply_at_the_band_counts_where_its_shape_changes(nb):
         h.apply(x)
         out.append(x)
     assert float((out[0] - out[1]).abs().max()) < 1e-12 * float(out[0].abs().max())
+
+
+@pytest.mark.parametrize("dtype,which,tol", [(torch.complex128, 2, 1e-12), (torch.complex64, 3, 1e-6)])
+def test_every_apply_variant_on_a_large_call(dtype, which, tol):
+    """Small calls run one shape whatever the variant; here every colour is large enough for the shape asked for, with
+    a ragged last group, against native FP64 on the same states."""
+    s = _system(48)
+    nb = _apply_bands(s, 37)
+    psi = _random_states(s, nb, seed=13).to(dtype)
+    f = torch.rand(s.nk, 1, nb, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda", dtype=torch.float64) / nb
+    h = dftu.handle_for_system(s, nb)
+    for I in range(3):
+        h.set_u(I, 0.4, 0.05)
+    h.set_f64_mode(dftu.F64_NATIVE)
+    ref = psi.to(torch.complex128, copy=True)
+    h.project(ref)
+    h.occupations(f)
+    h.acbn0_uj()
+    h.apply(ref)
+    h.set_f64_mode(dftu.F64_PAIR)
+    top = float(ref.abs().max())
+    for variant in range(h.lib.dftu_kernel_variants(which)):
+        h.set_kernel_variant(which, variant)
+        x = psi.clone()
+        h.apply(x)
+        assert float((x.to(torch.complex128) - ref).abs().max()) < tol * top, variant
