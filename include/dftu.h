@@ -283,12 +283,12 @@ dftu_status dftu_project_sphere_noalloc(const void* psi, dftu_prec prec, int nba
                                         const int32_t* idx, const double* phase, const double* phi, int npts,
                                         int M, double dV, double* p_out, dftu_stream stream);
 
-/* The memory-system ceiling of the access pattern, for roofline comparisons: one pass that reads every
+/* The access pattern alone with plain loads, a reference for roofline comparisons: one pass that reads every
  * sphere point of the first nbands states once (rmw = 0, the gather of dftu_project) or reads and writes
  * each back unchanged (rmw = 1, the read-modify-write of dftu_apply), with the same tiles and no
  * arithmetic.  The states' values are not changed.  Not part of the method (the paper has no counterpart);
- * the time of one pass bounds a projection and an apply with plain loads on this GPU (the complex64 projection
- * fetches smaller blocks and can pass it).  Asynchronous on stream. */
+ * a projection and an apply with plain loads cannot be faster on this GPU; other loads can (the complex64
+ * projection fetches smaller blocks and passes it).  Asynchronous on stream. */
 dftu_status dftu_access_ceiling(dftu_handle h, void* psi, dftu_prec prec, int nbands, int64_t ld_band, int rmw,
                                 dftu_stream stream);
 

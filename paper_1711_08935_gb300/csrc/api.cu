@@ -495,7 +495,7 @@ dftu_status dftu_setup_atoms(dftu_handle h, int natoms, const dftu_atom* atoms, 
     if (e == cudaSuccess) e = dalloc(c, &v.phi_hi, (size_t)phi_off);
     if (e == cudaSuccess) e = dalloc(c, &v.phi_lo, (size_t)phi_off);
     if (e == cudaSuccess) e = dalloc(c, &v.p, (size_t)rowsP * c->max_bands * MT);
-    v.part_dir_stride = (int64_t)rowsP * c->max_bands * TM;   // three slices: the current's three directions
+    v.part_dir_stride = (int64_t)rowsP * c->max_bands * TM;   // three slices: the tables of the current
     if (e == cudaSuccess) e = dalloc(c, &v.part, (size_t)3 * v.part_dir_stride);
     if (e == cudaSuccess) e = dalloc(c, &v.pgrad, (size_t)3 * rowsP * c->max_bands * MT);
     if (e == cudaSuccess) e = dalloc(c, &c->d_forces, (size_t)3 * natoms);

@@ -1,9 +1,9 @@
-// The memory-system ceiling of the projector's access pattern: every sphere point of every state read
+// The projector's access pattern alone, a reference for the kernels' rates: every sphere point of every state read
 // once (the projection's gather), or read and written back unchanged (the apply's read-modify-write),
 // with no arithmetic.  The tiles, grid order and lanes per band are those of the streaming kernels, so
-// the time of one pass bounds what the projection and the apply can reach on this GPU; roofline
-// fractions are quoted against it beside the copy bandwidth.  Plain loads: the complex64 projection, whose loads fetch
-// 64-byte blocks instead of whole lines, can run above it.
+// the time of one pass is a reference for the projection and the apply on this GPU, quoted beside the
+// copy bandwidth.  It is that of plain loads, not a bound: the complex64 projection, whose loads fetch 64-byte blocks
+// instead of whole lines, runs above it.
 #include "dftu_internal.cuh"
 
 namespace dftu {

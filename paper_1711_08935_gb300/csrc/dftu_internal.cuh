@@ -116,10 +116,10 @@ struct View {
     double2* seg_phase;    // [nseg][nk] exp(+i k.T)
 
     double2* p;            // [nk*ns][max_bands][MT]
-    double2* pgrad;        // [3][nk*ns][max_bands][MT] projections of the state gradients (forces)
-    double2* part;         // [3][nk*ns][max_bands][TM]: one slice per direction of a three-table projection
-    int64_t phi_dir_stride;    // elements between the orbital tables of successive directions (0: one table)
-    int64_t part_dir_stride;   // elements between the partial-sum slices of successive directions
+    double2* pgrad;        // [3][nk*ns][max_bands][MT] projections of the state gradients (forces), or onto the tables of the current
+    double2* part;         // [3][nk*ns][TM][max_bands]: one slice per table of a projection onto several
+    int64_t phi_dir_stride;    // elements between successive orbital tables (0: one table)
+    int64_t part_dir_stride;   // elements between the partial-sum slices of successive tables
     double* nbar;          // collinear [nk*ns][max_bands][nspecies]; non-collinear [nk][max_bands][nspecies]
     double2* rho;          // per atom: collinear [ns][M][M]; non-collinear [2M][2M]   (rho = n^T)
     double2* pbar;         // same layout, renormalised (Eq. 8), transposed like rho

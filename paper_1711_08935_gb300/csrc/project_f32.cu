@@ -6,10 +6,8 @@ namespace dftu {
 // The shapes selectable with dftu_set_kernel_variant, listed once for the single-system and the batched
 // launches: X(variant, policy, lanes per band Q, points per chain, band groups per CTA, L2 prefetch,
 // minimum blocks per SM, threads per CTA, tile size).  Variant 0 is the default case of each switch.
-// P_F32B2 is the complex64 form with two bands per lane, P_F32B2F the same with each product's hi and lo
-// halves folded into one sum, P_F32 one band per lane.  PAIR L2 prefetch: 1 = the next chain, 5 = also
-// the next band's first chain.  Tile size PTILE selects the projection's own tiling (single-system
-// launches; batched launches use TILE, on which PAIR variant 1 is the default shape).
+// P_F32B2 has two bands per lane, P_F32B2F also each product's hi and lo halves folded into one sum, P_F32 one band
+// per lane.  Tile size PTILE selects the projection's own tiling (single-system launches).
 #define DFTU_PROJECT_SHAPES_F32(X) \
     X(1, P_F32B2F, 16, 8, 4, 0, 3, 256, PTILE) X(2, P_F32B2F, 8, 8, 4, 0, 3, 256, TILE) X(3, P_F32B2, 8, 8, 4, 0, 2, 256, TILE) \
     X(4, P_F32B2F, 16, 8, 4, 0, 2, 256, TILE) X(5, P_F32B2F, 16, 8, 8, 0, 3, 256, TILE) \

@@ -31,7 +31,7 @@ namespace dftu {
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
-struct DF2 { float2 h, l; };
+struct DF2 { float2 h, l; };   // (re, im) pair of double-float numbers
 
 // Gather of one complex64 state value, 0 where !in (predicated, no branch).  The 64-byte prefetch size makes
 // L2 fetch the 64-byte blocks that hold a run of points instead of whole 128-byte lines (1.31x instead of
@@ -46,7 +46,7 @@ __device__ __forceinline__ float2 ld_gather(const float2* p, bool in) {
 }
 
 // Ask L2 to start fetching a line a later chain will read (no register is held for it).
-__device__ __forceinline__ void prefetch_l2(const void* ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr)); }   // (re, im) pair of double-float numbers
+__device__ __forceinline__ void prefetch_l2(const void* ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr)); }
 
 // TwoSum(a.h, b.h) with the low parts added: a <- a + b.
 __device__ __forceinline__ void df_add(DF2& a, const DF2& b) {
@@ -69,7 +69,7 @@ __device__ __forceinline__ float pow2f(int e) {   // 2^e as float for e in [-126
 
 // Tile partial sum, before the Bloch phase and dV (k_tile_reduce applies both once per image segment).
 // Layout [k*spin][tile slot (moff + m)][band], band fastest, so the reduce reads 32 bands of one slot in
-// one coalesced access.  poff: offset of the direction's slice (three-table projections), 0 otherwise.
+// one coalesced access.  poff: offset of the table's slice (projections onto several tables), 0 otherwise.
 __device__ __forceinline__ void write_partial(const View& v, const Tile& t, int ks, int band, int m, double re, double im,
                                               int64_t poff) {
     v.part[poff + ((int64_t)ks * v.TM + t.moff + m) * v.max_bands + band] = make_double2(re, im);

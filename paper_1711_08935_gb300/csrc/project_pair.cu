@@ -3,19 +3,14 @@
 
 namespace dftu {
 
-// The shapes selectable with dftu_set_kernel_variant, listed once for the single-system and the batched
-// launches: X(variant, policy, lanes per band Q, points per chain, band groups per CTA, L2 prefetch,
-// minimum blocks per SM, threads per CTA, tile size).  Variant 0 is the default case of each switch.
-// P_F32B2 is the complex64 form with two bands per lane, P_F32B2F the same with each product's hi and lo
-// halves folded into one sum, P_F32 one band per lane.  PAIR L2 prefetch: 1 = the next chain, 5 = also
-// the next band's first chain.  Tile size PTILE selects the projection's own tiling (single-system
-// launches; batched launches use TILE, on which PAIR variant 1 is the default shape).
+// The shapes selectable with dftu_set_kernel_variant: X as for the complex64 shapes (project_f32.cu).  L2 prefetch: 1 =
+// the next chain, 5 = also the next band's first chain.  Tile size PTILE selects the projection's own tiling
+// (single-system launches; batched launches use TILE, on which variant 1 is the default shape).
 #define DFTU_PROJECT_SHAPES_PAIR(X) \
     X(1, P_PAIR, 8, 8, 8, 5, 2, 256, TILE) X(2, P_PAIR, 8, 8, 4, 5, 2, 256, PTILE) X(3, P_PAIR, 8, 8, 16, 5, 2, 256, PTILE) \
     X(4, P_PAIR, 16, 8, 16, 5, 2, 256, PTILE) X(5, P_PAIR, 8, 8, 8, 1, 2, 256, PTILE) X(6, P_PAIR, 8, 8, 4, 5, 2, 256, TILE) \
     X(7, P_PAIR, 8, 6, 8, 5, 2, 256, PTILE)
 #define DFTU_PROJECT_DEFAULT_PAIR P_PAIR, 8, 8, 8, 5, 2, 256, PTILE
-
 
 // The default shape, with fewer bands per CTA where the grid would not fill the GPU (balanced_groups).  Calls so
 // small that single groups on the 1024-point tiles do not fill the GPU are one chain of latencies per CTA: they
