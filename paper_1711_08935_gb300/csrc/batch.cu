@@ -162,7 +162,6 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
         }
         args[s] = a;
         max_reduce = std::max<int64_t>(max_reduce, (int64_t)c->nk * c->ns * nbands[s] * c->MT);
-        max_ctas = std::max<int64_t>(max_ctas, (int64_t)c->nk * c->ns * ((nbands[s] + 31) / 32) * (int64_t)c->atoms.size());
         max_rows = std::max(max_rows, (c->spin == DFTU_NONCOLLINEAR ? c->nk : c->nk * c->ns) * nbands[s] * c->nspecies);
     }
     // The persistent kernels take items in list order; a member's items all take its bound bands, so the members with the
@@ -177,6 +176,7 @@ dftu_status dftu_batch_bind(dftu_batch b, const void* const* psi, dftu_prec prec
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
+    for (int s = 0; s < n; ++s) max_ctas = std::max(max_ctas, tile_reduce_blocks(b->members[s]->v, nbands[s]));
     b->bound = false;   // until the new tables stand
     free_tables(b);
     cudaError_t e = cudaSuccess;

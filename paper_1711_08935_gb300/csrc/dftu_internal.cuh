@@ -216,7 +216,7 @@ struct BatchLaunch {
     int nsys;
     int maxM;
     int64_t max_reduce;       // max over systems of (k*spin rows) * nbands * sum M
-    int64_t max_reduce_ctas;  // max over systems of (k*spin rows) * band chunks of 32 * atoms (the tile reduce's CTAs)
+    int64_t max_reduce_ctas;  // max over systems of the tile reduce's CTAs (tile_reduce_blocks)
     int max_rows_nbar;        // max over systems of rows * nbands * species (the Nbar threads)
     int max_atoms, max_ns;
 };
@@ -294,6 +294,9 @@ bool smem_configured(const void* fn, int bytes);
 
 // SMs of the current device (looked up once per device).
 int sm_count();
+
+// CTAs of a tile reduce over nbands bands on the current device, in the form it takes at that size.
+int64_t tile_reduce_blocks(const View& v, int nbands);
 
 #ifdef __CUDACC__
 // The kernels of a step run back to back on one stream, many of them for a few microseconds.  Launched dependently, a

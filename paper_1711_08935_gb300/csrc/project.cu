@@ -104,7 +104,7 @@ __device__ __forceinline__ void reduce_atom(const View& v, int nbands, int ks, i
 }
 
 // CTAs of one system's reduce: (k*spin, band chunk, atom), atoms fastest.
-static int64_t reduce_ctas(const View& v, int nbands) { return (int64_t)v.nk * v.ns * ((nbands + RED_BANDS - 1) / RED_BANDS) * v.natoms; }
+__host__ __device__ static int64_t reduce_ctas(const View& v, int nbands) { return (int64_t)v.nk * v.ns * ((nbands + RED_BANDS - 1) / RED_BANDS) * v.natoms; }
 
 __device__ __forceinline__ void reduce_item(const View& v, int nbands, int64_t id, int table, int64_t p_stride) {
     __shared__ double2 sm[RED_SLICES * MAXM * RED_LD];
@@ -127,62 +127,40 @@ __global__ void __launch_bounds__(CTA, 2) k_tile_reduce(View v, int nbands) {
     reduce_item(v, nbands, blockIdx.x, 0, 0);
 }
 
-// The same sums in the same order with a thread per (k*spin, orbital, band), band fastest, walking the atom's tiles
-// range by range: a state's bits do not depend on the size of the call, nor on whether it runs in a batch (which takes
-// the form above).  Where that form takes more than two waves, the SMs are full either way and this one holds more
-// warps: 512 CTAs of the form above 37 (this) against 33 us, 1024 CTAs 31 against 40, 2048 CTAs 64 against 84 (measured
-// with one sum per atom; the ranges changed whole projections of 1024 and 2048 oxide states by -4 and +3 us).
-__global__ void k_tile_reduce_states(View v, int nbands) {
-    dependent_release();
-    dependent_wait();
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The same sums with a thread per (k*spin, orbital, band), band fastest, walking the atom's tiles in order.  Where the
+// form above takes more than two waves, the SMs are full either way and this one holds more warps: 512 CTAs of the form
+// above 37 (this) against 33 us, 1024 CTAs 31 against 40, 2048 CTAs 64 against 84.  (In the ranges of the form above,
+// for one order at every size, it is bound by the instructions that close them: 64 atoms, 2048 states 100 -> 130 us.)
+__device__ __forceinline__ void reduce_state(const View& v, int nbands, int64_t g) {
     if (g >= (int64_t)v.nk * v.ns * v.MT * nbands) return;
     const int band = (int)(g % nbands), j = (int)(g / nbands % v.MT), ks = (int)(g / nbands / v.MT);
-    const int a = v.orb_atom[j], m = j - v.atom_moff[a], M = v.atom_M[a];
-    const int t0 = v.atom_tile_beg[a], t1 = v.atom_tile_end[a], per = (t1 - t0 + RED_SLICES - 1) / RED_SLICES;
-    const double2* part = v.part + ((int64_t)ks * v.TM + v.tiles[t0].moff + m) * v.max_bands + band;
+    const int a = v.orb_atom[j], m = j - v.atom_moff[a];
+    const double2* part = v.part + ((int64_t)ks * v.TM + m) * v.max_bands + band;
     const double2* phase = v.seg_phase + ks / v.ns;
-    double2 sum = make_double2(0.0, 0.0), range = sum, in_seg = sum;
-    int seg = v.tiles[t0].seg, end = t0 + per;   // open segment; end of the open range
-    double2 ph = phase[(int64_t)seg * v.nk];
-    constexpr int B = 6;                         // tiles in flight
-    for (int t = t0; t < t1; t += B) {
-        double2 x[B];
-        int sg[B];
-#pragma unroll
-        for (int u = 0; u < B; ++u) {
-            const bool on = t + u < t1;
-            sg[u] = on ? v.tiles[t + u].seg : -1;
-            x[u] = on ? part[(int64_t)(t + u - t0) * M * v.max_bands] : make_double2(0.0, 0.0);
+    double2 sum = make_double2(0.0, 0.0), in_seg = sum;
+    int seg = -1;
+    for (int t = v.atom_tile_beg[a]; t < v.atom_tile_end[a]; ++t) {
+        const Tile& tl = v.tiles[t];
+        if (tl.seg != seg) {
+            if (seg >= 0) add_segment(sum, phase[(int64_t)seg * v.nk], in_seg);
+            seg = tl.seg;
+            in_seg = make_double2(0.0, 0.0);
         }
-#pragma unroll
-        for (int u = 0; u < B; ++u) {
-            if (t + u >= t1) break;
-            if (sg[u] != seg || t + u == end) {
-                add_segment(range, ph, in_seg);
-                in_seg = make_double2(0.0, 0.0);
-                if (sg[u] != seg) {
-                    seg = sg[u];
-                    ph = phase[(int64_t)seg * v.nk];
-                }
-                if (t + u == end) {
-                    sum.x += range.x;
-                    sum.y += range.y;
-                    range = make_double2(0.0, 0.0);
-                    end += per;
-                }
-            }
-            in_seg.x += x[u].x;
-            in_seg.y += x[u].y;
-        }
+        const double2 x = part[(int64_t)tl.moff * v.max_bands];
+        in_seg.x += x.x;
+        in_seg.y += x.y;
     }
-    add_segment(range, ph, in_seg);
-    sum.x += range.x;
-    sum.y += range.y;
+    add_segment(sum, phase[(int64_t)seg * v.nk], in_seg);
     sum.x *= v.dV;
     sum.y *= v.dV;
     if (!isfinite(sum.x) || !isfinite(sum.y)) atomicOr(v.status, ST_NONFINITE);
     v.p[((int64_t)ks * v.max_bands + band) * v.MT + j] = sum;
+}
+
+__global__ void k_tile_reduce_states(View v, int nbands) {
+    dependent_release();
+    dependent_wait();
+    reduce_state(v, nbands, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // The tables of the current (blockIdx.y) in one launch, each into its slice of p.
@@ -190,8 +168,20 @@ __global__ void __launch_bounds__(CTA, 2) k_tile_reduce_tables(View v, int nband
     if ((int)blockIdx.y < cur_tables(v.atom_M[blockIdx.x % v.natoms])) reduce_item(v, nbands, blockIdx.x, blockIdx.y, p_stride);
 }
 
-__global__ void __launch_bounds__(CTA, 2) k_tile_reduce_batch(const View* __restrict__ views, const ProjArgs* __restrict__ args) {
-    reduce_item(views[blockIdx.y], args[blockIdx.y].nbands, blockIdx.x, 0, 0);
+// Every member in the form that the same call made alone takes (states_above: reduce_by_states), so that it gets the same bits.
+__global__ void __launch_bounds__(CTA, 2) k_tile_reduce_batch(const View* __restrict__ views, const ProjArgs* __restrict__ args, int64_t states_above) {
+    const View& v = views[blockIdx.y];
+    const int nbands = args[blockIdx.y].nbands;
+    if (reduce_ctas(v, nbands) > states_above) reduce_state(v, nbands, (int64_t)blockIdx.x * CTA + threadIdx.x);
+    else reduce_item(v, nbands, blockIdx.x, 0, 0);
+}
+
+// The thread-per-state form above this many CTAs of the other: two waves (two CTAs per SM).
+static int64_t reduce_by_states() { return 4 * (int64_t)sm_count(); }
+
+int64_t tile_reduce_blocks(const View& v, int nbands) {
+    const int64_t ctas = reduce_ctas(v, nbands);
+    return ctas > reduce_by_states() ? ((int64_t)v.nk * v.ns * v.MT * nbands + CTA - 1) / CTA : ctas;
 }
 
 // Whether MINB CTAs of fn with smem bytes of dynamic shared memory fit on one SM (cached per kernel and size).
@@ -255,11 +245,8 @@ cudaError_t launch_project_c64_tiles(const View& sub, const void* psi, int nband
 }
 
 cudaError_t launch_tile_reduce(const View& v, int nbands, cudaStream_t st) {
-    if (reduce_ctas(v, nbands) > 4 * (int64_t)sm_count()) {
-        const int64_t n = (int64_t)v.nk * v.ns * v.MT * nbands;
-        return launch_dependent(k_tile_reduce_states, (unsigned)((n + CTA - 1) / CTA), CTA, 0, st, v, nbands);
-    }
-    return launch_dependent(k_tile_reduce, (unsigned)reduce_ctas(v, nbands), CTA, 0, st, v, nbands);
+    auto fn = reduce_ctas(v, nbands) > reduce_by_states() ? k_tile_reduce_states : k_tile_reduce;
+    return launch_dependent(fn, (unsigned)tile_reduce_blocks(v, nbands), CTA, 0, st, v, nbands);
 }
 
 cudaError_t launch_project_dirs(const View& v, const void* psi, dftu_prec prec, dftu_f64_mode mode, int nbands,
@@ -284,7 +271,7 @@ cudaError_t launch_project_batch(const BatchLaunch& b, dftu_prec prec, dftu_f64_
     else if (mode == DFTU_F64_NATIVE) e = run_project_batch<P_F64, 8, 1, 4, 0>(b, st);
     else e = project_pair_batch(b, variant, st);
     if (e != cudaSuccess) return e;
-    k_tile_reduce_batch<<<dim3((unsigned)b.max_reduce_ctas, b.nsys), CTA, 0, st>>>(b.views, b.args);
+    k_tile_reduce_batch<<<dim3((unsigned)b.max_reduce_ctas, b.nsys), CTA, 0, st>>>(b.views, b.args, reduce_by_states());
     return cudaGetLastError();
 }
 

@@ -16,7 +16,7 @@ namespace dftu {
 
 // The default shape, with fewer bands per CTA where the grid would not fill the GPU (balanced_groups): lanes and
 // tiles stay, so the order of the FP32 sums does not depend on the size of the call and batched launches give
-// the same bits (the tile reduce keeps its order too).
+// the same bits (their tile reduce takes each member in the form that a single call of its size takes).
 cudaError_t project_f32(const View& v, const ProjArgs& a, int variant, cudaStream_t st, View* used) {
 #define DFTU_CASE(i, POL, Q, CH, NBG, PF, MB, NT, TP) case i: return run_project<POL, Q, CH, NBG, PF, MB, 0, 1, NT, TP>(v, a, st, used);
     switch (variant) {

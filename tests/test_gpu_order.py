@@ -1,4 +1,4 @@
-"""Orders that do not depend on the size of a call: wide members of a batch against the same calls made alone."""
+"""Members of a batch against the same calls made alone, bit for bit, at every size."""
 import numpy as np
 import pytest
 import torch
